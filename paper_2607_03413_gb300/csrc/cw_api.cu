@@ -956,6 +956,10 @@ cw_status cw_op_create(cw_mesh mh, int degree, int kind, int geom, int prec, int
     op->mesh = m;
     op->p = degree;
     op->n = degree + 1;
+    if (geom == CW_GEOM_METRIC) {  // the variant to start with
+        if (prec == CW_PREC_F64) op->stage = default_stage(op->n, false);
+        if (default_cells(op->n, prec_f32_arith(prec), vec_elem_size(prec) == 4)) op->cpb = tile_cells(op->n, true) / 2;
+    }
     op->kind = kind;
     op->geom = geom;
     op->prec = prec;

@@ -35,8 +35,8 @@ namespace cw {
 // This halves the multiply-adds of a line contraction (Kronbichler and Kormann's even-odd
 // decomposition for sum factorisation).
 // For double-float tables the same entries are also stored lane-paired, P[a][b] = (E[a][b], O[a][b])
-// and PM[a] = (Mid[a], 0), so that the even and odd sums of an output pair run as one paired
-// multiply-add chain with each coefficient pair one 64-bit constant operand.
+// so that the even and odd sums of an output pair run as one paired multiply-add chain with each
+// coefficient pair one 64-bit constant operand; FP32 tables also hold PM[a] = (Mid[a], 0).
 template <class C>
 struct EOPair {
     struct type {};
@@ -57,7 +57,7 @@ struct EOMat {
     C O[NA][H > 0 ? H : 1];
     C Mid[NA];
     typename EOPair<C>::type P[NA][H > 0 ? H : 1];
-    typename EOPair<C>::type PM[NA];
+    typename EOPair<C>::type PM[std::is_same<C, float>::value ? NA : 1];
 };
 
 template <int N, class C>
@@ -124,36 +124,39 @@ __device__ __forceinline__ void contract_eo(const EOMat<N, typename Ar::C> &M, c
 {
     using T = typename Ar::T;
     constexpr int H = N / 2;
+    // double-float at N = 3: everything renormalised (83 operations per line instead of 68), which makes
+    // the form as accurate as the full one with renormalised outputs (93 operations)
+    constexpr bool N3 = N == 3 && std::is_same<Ar, ArDF>::value;
     T e[H], o[H];
 #pragma unroll
     for (int b = 0; b < H; ++b) {
         e[b] = Ar::add(in[b], in[N - 1 - b]);
         o[b] = Ar::sub(in[b], in[N - 1 - b]);
+        if constexpr (N3) e[b] = Ar::norm(e[b]), o[b] = Ar::norm(o[b]);
     }
     if constexpr (std::is_same<Ar, ArDF>::value) {
         // Double-float: the even and odd sums of an output pair run as one chain of paired FP32
-        // operations (lane x even, lane y odd; the middle term enters lane y multiplied by 0, which
-        // leaves it unchanged), each lane bit-identical to the scalar chain. (Pairing the e/o
+        // operations (lane x even, lane y odd), each lane bit-identical to the scalar chain; the middle
+        // input of an odd N enters the even sum only, as a scalar operation on lane x. (Pairing the e/o
         // formation and the final add/subtract as well was slower: the lane shuffles cost more.)
         df64p eo[H];
 #pragma unroll
         for (int b = 0; b < H; ++b) eo[b] = dfp_pack(e[b], o[b]);
-        df64p xm;
-        if constexpr (N % 2 == 1) xm = dfp_pack(in[H], in[H]);
 #pragma unroll
         for (int a = 0; a < H; ++a) {
             df64p y2 = dfp_mul(eo[0], M.P[a][0]);
 #pragma unroll
             for (int b = 1; b < H; ++b) dfp_mad(y2, eo[b], M.P[a][b]);
-            if constexpr (N % 2 == 1) dfp_mad(y2, xm, M.PM[a]);
-            const T ye = dfp_x(y2), yo = dfp_y(y2);
+            T ye = dfp_x(y2);
+            const T yo = dfp_y(y2);
+            if constexpr (N % 2 == 1) Ar::mad(ye, in[H], M.Mid[a]);
             // without NRM the outputs stay unnormalised (|lo| a few ulp of hi): every consumer is a
             // double-float operation or the final conversion, which take that form as it is
             const T sum = Ar::add(ye, yo);
-            out[a] = NRM ? Ar::norm(sum) : sum;
+            out[a] = NRM || N3 ? Ar::norm(sum) : sum;
             const T d = Ar::sub(ye, yo);
             const T dd = S > 0 ? d : Ar::neg(d);
-            out[N - 1 - a] = NRM ? Ar::norm(dd) : dd;
+            out[N - 1 - a] = NRM || N3 ? Ar::norm(dd) : dd;
         }
     } else if constexpr (std::is_same<Ar, ArF32>::value) {
         // FP32: the same pairing with FFMA2 (lane x even, lane y odd)
@@ -192,22 +195,23 @@ __device__ __forceinline__ void contract_eo(const EOMat<N, typename Ar::C> &M, c
             T ye = Ar::mul(in[H], M.Mid[H]);
 #pragma unroll
             for (int b = 0; b < H; ++b) Ar::mad(ye, e[b], M.E[H][b]);
-            out[H] = NRM ? Ar::norm(ye) : ye;
+            out[H] = NRM || N3 ? Ar::norm(ye) : ye;
         } else {
             T yo = Ar::mul(o[0], M.O[H][0]);
 #pragma unroll
             for (int b = 1; b < H; ++b) Ar::mad(yo, o[b], M.O[H][b]);
-            out[H] = NRM ? Ar::norm(yo) : yo;
+            out[H] = NRM || N3 ? Ar::norm(yo) : yo;
         }
     }
 }
 
-// line contraction with B, B^T, D or D^T: even-odd form from N = 4 up, full form below
+// line contraction with B, B^T, D or D^T: even-odd form from N = 4 up (in double-float from N = 3), full
+// form below
 template <int N, class Ar, int WHICH, bool NRM = true>  // WHICH: 0 B, 1 B^T, 2 D, 3 D^T
 __device__ __forceinline__ void sweep(const TabMetric<N, typename Ar::C> &tab, const typename Ar::T (&in)[N],
                                       typename Ar::T (&out)[N])
 {
-    if constexpr (N >= 4) {
+    if constexpr (N >= (std::is_same<Ar, ArDF>::value ? 3 : 4)) {
         if constexpr (WHICH == 0) contract_eo<N, 1, Ar, NRM>(tab.Bf, in, out);
         else if constexpr (WHICH == 1) contract_eo<N, 1, Ar, NRM>(tab.Bt, in, out);
         else if constexpr (WHICH == 2) contract_eo<N, -1, Ar, NRM>(tab.Df, in, out);
@@ -353,11 +357,30 @@ __host__ __device__ constexpr int metric_ncomp(int kind) { return kind == 1 ? 6 
 // TMA, metric tile prefetched into L2 by a bulk prefetch (a third of the shared memory of mode 1,
 // so more CTAs per SM), then read with direct loads; 3: the metric tile already in shared memory
 // (staged by the caller for several right-hand sides, gsm), x read directly.
+// Line buffers of metric_tile: three for 4-byte elements; two for 8-byte ones (double-float and FP64
+// arithmetic), whose y-derivatives go back into buffer 0 after one more barrier: with the metric staged
+// a CTA then needs 72 instead of 80 bytes of shared memory per value (K+M), which is one more CTA per SM
+// at n = 5 and 8 (3 instead of 2).
+template <class T>
+constexpr int line_buffers()
+{
+    return sizeof(T) == 8 ? 2 : 3;
+}
+
+// Stage 2 in double-float arithmetic: each thread copies the metric entries of its own pencil into a
+// private ring of kRing points in shared memory with 8-byte cp.async, kRing points ahead of their use.
+constexpr int kRing = 2;
+template <class Ar, int STAGE, bool RC>
+constexpr bool metric_ring()
+{
+    return std::is_same<Ar, ArDF>::value && STAGE == 2 && !RC;
+}
+
 template <int N, int CPB, class T, class GS, bool REMAP = true>
 __host__ __device__ constexpr size_t metric_smem_bytes(int nc, int stage)
 {
-    constexpr size_t lb = 3 * TileLines<N, CPB, sizeof(T), REMAP>::RS * sizeof(T);  // a multiple of 16
-    return stage == 1 ? lb + (CPB * nc * N * N * N * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 : lb;
+    constexpr size_t lb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), REMAP>::RS * sizeof(T);  // a multiple of 16
+    return stage == 1 ? lb + (CPB * nc * N * N * N * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 + (std::is_same<T, df64>::value ? kRing * nc * N * N * CPB * sizeof(GS) : 0) : lb;
 }
 
 // One tile of `cpt` consecutive cells starting at cell tile*cpt, worked by CPB cell slots of N*N
@@ -416,6 +439,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
     using TL = TileLines<N, CPB, sizeof(T), REMAP>;
     static_assert(line_map_is_bijection<N, CPB, sizeof(T), REMAP>(), "every line has one thread");
     constexpr int N2 = N * N, N3 = N2 * N, PI = TL::PI, PP = TL::PP, CS = TL::CS, RS = TL::RS;
+    constexpr int NB = line_buffers<T>(), YB = NB == 3 ? 2 : 0;  // YB: the buffer of the y-derivatives
     const bool HAS_K = (kind & 1) != 0, HAS_M = (kind & 2) != 0;
     const int NC = metric_ncomp(kind);
     T *S0 = reinterpret_cast<T *>(smem_raw);
@@ -445,7 +469,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
     uint64_t *bar = nullptr;
     const uint32_t lim = dbg_extra ? kWaitLimitInjected : kWaitLimit;
     if constexpr (STAGE == 1) {
-        const size_t offg = 3 * RS * sizeof(T);
+        const size_t offg = NB * RS * sizeof(T);
         GS *sG = reinterpret_cast<GS *>(smem_raw + offg);
         bar = reinterpret_cast<uint64_t *>(smem_raw + offg + (CPB * NC * N3 * sizeof(GS) + 15) / 16 * 16);
         VS *sX = reinterpret_cast<VS *>(S0 + RS);  // buffer 1 is free until the gradients
@@ -480,7 +504,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         gs = gsm + (act ? c : 0) * NC * N3;
         g_smem = true;
     } else if constexpr (STAGE == 2) {
-        bar = reinterpret_cast<uint64_t *>(smem_raw + 3 * RS * sizeof(T));
+        bar = reinterpret_cast<uint64_t *>(smem_raw + NB * RS * sizeof(T));
         VS *sX = reinterpret_cast<VS *>(S0 + RS);
         const VS *xsrc = x + cell0 * N3;
         constexpr int GV = RC ? kTriCoef : 0;  // geometry values per cell (RC), else NC * N3
@@ -504,6 +528,27 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         }
     }
 
+    // RING: this thread's ring of the metric entries of its next kRing points
+    constexpr bool RING = metric_ring<Ar, STAGE, RC>();
+    constexpr int T1 = N2 * CPB;
+    [[maybe_unused]] GS *ring = reinterpret_cast<GS *>(smem_raw + NB * RS * sizeof(T) + 16) + t;
+    [[maybe_unused]] const GS *gring = geo + (act ? cell : 0) * NC * N3 + r;
+    auto ring_issue = [&](int k) {
+        if (k < N) {
+            GS *d = ring + (k % kRing) * NC * T1;
+            const GS *g = gring + N2 * k;
+            if (HAS_K) {
+#pragma unroll
+                for (int i = 0; i < 6; ++i) cp_async8(d + i * T1, g + i * N3);
+            }
+            if (HAS_M) cp_async8(d + (NC - 1) * T1, g + (NC - 1) * N3);
+        }
+        cp_async_commit();  // one group per point, empty past the end
+    };
+    if constexpr (RING) {
+#pragma unroll
+        for (int k = 0; k < kRing; ++k) ring_issue(k);
+    }
     {
         T v[N], w[N], u[N], acc[N], gx[N], gy[N], gz[N];
         // (1) x-line (j,k) = (ra, rb): N contiguous values of the cell, contracted with B along x
@@ -545,12 +590,13 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                 CW_TST(1, xo, 1, w);
                 CW_TLD(0, yo, PI, v);
                 sweep<N, Ar, 2, NRM>(tab, v, w);
-                CW_TST(2, yo, PI, w);
+                if constexpr (NB == 2) __syncthreads();  // every line of buffer 0 has been read
+                CW_TST(YB, yo, PI, w);
             }
             __syncthreads();
             {
                 CW_TLD(1, zo, PP, gx);
-                CW_TLD(2, zo, PP, gy);
+                CW_TLD(YB, zo, PP, gy);
             }
         }
         // the metric tile's wait (a thread whose wait expired reads the metric from global memory)
@@ -604,6 +650,15 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
             for (int k = 0; k < N; ++k) {
                 const GS *g = gc + N2 * k;
                 T gxx, gyy, gzz, gxy, gxz, gyz, cmr;
+                if constexpr (RING) {
+                    cp_async_wait<kRing - 1>();  // the copies of point k have landed
+                    const GS *rg = ring + (k % kRing) * NC * T1;
+                    if (HAS_K) {
+                        gxx = Ar::from(rg[0 * T1]), gyy = Ar::from(rg[1 * T1]), gzz = Ar::from(rg[2 * T1]);
+                        gxy = Ar::from(rg[3 * T1]), gxz = Ar::from(rg[4 * T1]), gyz = Ar::from(rg[5 * T1]);
+                    }
+                    if (HAS_M) cmr = Ar::from(rg[(NC - 1) * T1]);
+                }
                 if constexpr (RC) {
                     const T zeta = tab.xq[k];
                     T jx[3], jy[3];
@@ -649,7 +704,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                     }
                 }
                 if (HAS_K) {
-                    if constexpr (!RC) {
+                    if constexpr (!RC && !RING) {
                         gxx = Ar::from(g[0 * N3]), gyy = Ar::from(g[1 * N3]);
                         gzz = Ar::from(g[2 * N3]), gxy = Ar::from(g[3 * N3]);
                         gxz = Ar::from(g[4 * N3]), gyz = Ar::from(g[5 * N3]);
@@ -671,11 +726,12 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                     gz[k] = NRM ? Ar::norm(hz) : hz;
                 }
                 if (HAS_M) {
-                    if constexpr (!RC) cmr = Ar::from(g[(NC - 1) * N3]);
+                    if constexpr (!RC && !RING) cmr = Ar::from(g[(NC - 1) * N3]);
                     const T cm = cmr;
                     acc[k] = NRM ? Ar::norm(Ar::mul(u[k], cm)) : Ar::mul(u[k], cm);
                     if constexpr (DOT) df_mad(*dot, Ar::to_df(u[k]), Ar::to_df(acc[k]));  // c u^2
                 }
+                if constexpr (RING) ring_issue(k + kRing);  // into the slot point k was read from
             }
         }
         if (HAS_K) {
@@ -684,22 +740,22 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                 sweep<N, Ar, 3, NRM>(tab, gz, v);
 #pragma unroll
                 for (int k = 0; k < N; ++k) acc[k] = HAS_M ? Ar::add(acc[k], v[k]) : v[k];
-                CW_TST(1, zo, PP, gx);  // own pencil only: no other thread reads s1/s2 pencils now
-                CW_TST(2, zo, PP, gy);
+                CW_TST(1, zo, PP, gx);  // own pencil only: no other thread reads these pencils now
+                CW_TST(YB, zo, PP, gy);
             }
             __syncthreads();
             {
                 CW_TLD(1, xo, 1, v);
                 sweep<N, Ar, 3, NRM>(tab, v, w);
                 CW_TST(1, xo, 1, w);
-                CW_TLD(2, yo, PI, v);
+                CW_TLD(YB, yo, PI, v);
                 sweep<N, Ar, 3, NRM>(tab, v, w);
-                CW_TST(2, yo, PI, w);
+                CW_TST(YB, yo, PI, w);
             }
             __syncthreads();
             {
                 CW_TLD(1, zo, PP, v);
-                CW_TLD(2, zo, PP, w);
+                CW_TLD(YB, zo, PP, w);
 #pragma unroll
                 for (int k = 0; k < N; ++k) {
                     const T t = Ar::add(acc[k], Ar::add(v[k], w[k]));

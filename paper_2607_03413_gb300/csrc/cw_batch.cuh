@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
     __shared__ long long s_next;
     __shared__ int s_prob;
     // STAGE 1 layout: [line buffers][mbarrier, 16 B][metric tile]
-    const size_t offb = 3 * TileLines<N, CPB, sizeof(T), true>::RS * sizeof(T);  // a multiple of 16
+    const size_t offb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), true>::RS * sizeof(T);  // a multiple of 16
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + offb);
     GS *sG = reinterpret_cast<GS *>(smem_raw + offb + 16);
     if (threadIdx.x == 0) s_next = static_cast<long long>(atomicAdd(counter, 1ull));

@@ -30,6 +30,16 @@ __host__ __device__ constexpr int tile_cells(int n, bool f32)
            : n == 6 ? (f32 ? 8 : 4) : n == 7 ? (f32 ? 8 : 4) : 2;
 }
 
+// Staging mode a stored-metric operator starts with (op.stage). FP32 arithmetic: 1 (input and metric
+// tiles by TMA). Double-float: 1 or, where the metric tile's shared memory costs too many CTAs per SM,
+// 2 (each thread's metric entries two points ahead by 8-byte cp.async): Laplace at 51^3 Q5 866 us against
+// 985, 35^3 Q7 710 against 721, 64^3 Q4 K+M 817 against 823; at 78^3 Q3 565 against 533 and 42^3 Q6 857
+// against 784 mode 1 stays.
+__host__ __device__ constexpr int default_stage(int n, bool f32) { return !f32 && (n == 5 || n == 6 || n == 8) ? 2 : 1; }
+// Whether an operator starts with the alternative tile (half the default): FP32 vectors at n = 7, where
+// 8 cells are 2 CTAs per SM (42^3 Q6 Laplace 175 us with 4 cells, 281 with 8; BF16 182 with 8, 216 with 4).
+__host__ __device__ constexpr bool default_cells(int n, bool f32, bool vec4) { return f32 && n == 7 && vec4; }
+
 // whether a precision computes in FP32 arithmetic (its kernels use the FP32 tile sizes)
 __host__ __device__ inline bool prec_f32_arith(int prec)
 {

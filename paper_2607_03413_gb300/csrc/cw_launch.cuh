@@ -65,7 +65,6 @@ void fill_metric_tab(TabMetric<N, C> &t, const Tables1D &tb, MK mk)
             E.Mid[a] = mk((N % 2 == 1) ? M[a][H] : 0.0);
             if constexpr (std::is_same<C, df64>::value) {
                 for (int b = 0; b < (H > 0 ? H : 1); ++b) E.P[a][b] = pair(E.E[a][b], E.O[a][b]);
-                E.PM[a] = pair(E.Mid[a], df64{0.0f, 0.0f});
             }
             if constexpr (std::is_same<C, float>::value) {
                 for (int b = 0; b < (H > 0 ? H : 1); ++b) {
@@ -109,6 +108,13 @@ template <int N, class Ar>
 constexpr int cpb_alt()
 {
     return cpb_default<N, Ar>() / 2;
+}
+
+// the tile an operator starts with (default_cells): the default, or the alternative where it is faster
+template <int N, class Ar, class VS>
+constexpr int cpb_tuned()
+{
+    return default_cells(N, std::is_same<Ar, ArF32>::value, sizeof(VS) == 4) ? cpb_alt<N, Ar>() : cpb_default<N, Ar>();
 }
 
 template <class K>
@@ -193,17 +199,18 @@ cudaError_t launch_metric(const Op &op, const void *x, void *y, cudaStream_t s, 
     return cudaGetLastError();
 }
 
-// One fused smoothing sweep (smooth_metric_kernel): default tile, input tile staged by TMA and the
-// metric prefetched into L2 (stage 2); the x-interfaces inside tiles are averaged, *xfuse receives the
+// One fused smoothing sweep (smooth_metric_kernel): default tile, input tile staged by TMA and, where
+// the metric is stored, the arithmetic's default staging of it (FP32: prefetched into L2); the x-interfaces inside tiles are averaged, *xfuse receives the
 // tile size for the x pass between tiles.
 template <int N, class Ar, class VS, class GS, bool RC>
 cudaError_t launch_smooth(const Op &op, void *u, const void *b, const void *dhat, cudaStream_t s, int *xfuse)
 {
-    constexpr int CPB = cpb_default<N, Ar>();
+    constexpr int CPB = cpb_tuned<N, Ar, VS>();
+    constexpr int ST = RC || std::is_same<Ar, ArF32>::value ? 2 : default_stage(N, false);
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op.tab, [](double v) { return MakeC<Ar>::from(v); });
-    const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op.kind), 2);
-    auto kern = smooth_metric_kernel<N, CPB, Ar, VS, GS, 2, RC>;
+    const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op.kind), ST);
+    auto kern = smooth_metric_kernel<N, CPB, Ar, VS, GS, ST, RC>;
     static size_t opted[kMaxDevices] = {};
     if (cudaError_t e = ensure_smem(kern, smem, opted); e != cudaSuccess) return e;
     const unsigned grid = (unsigned)((op.E + CPB - 1) / CPB);
@@ -240,7 +247,7 @@ cudaError_t launch_smooth_degree(const Op &op, void *u, const void *b, const voi
 template <int N, class Ar, class VS, class GS, bool RC = false>
 cudaError_t launch_metric_dot(const Op &op, const void *x, void *y, double *part, int64_t *nblocks, cudaStream_t s)
 {
-    constexpr int CPB = cpb_default<N, Ar>(), ST = RC ? 2 : 1;
+    constexpr int CPB = cpb_tuned<N, Ar, VS>(), ST = RC ? 2 : default_stage(N, std::is_same<Ar, ArF32>::value);
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op.tab, [](double v) { return MakeC<Ar>::from(v); });
     const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op.kind), ST);
