@@ -355,8 +355,9 @@ __host__ __device__ constexpr int metric_ncomp(int kind) { return kind == 1 ? 6 
 // global loads instead.
 // STAGE 0: direct loads; 1: x and metric tiles staged in shared memory by TMA; 2: x tile staged by
 // TMA, metric tile prefetched into L2 by a bulk prefetch (a third of the shared memory of mode 1,
-// so more CTAs per SM), then read with direct loads; 3: the metric tile already in shared memory
-// (staged by the caller for several right-hand sides, gsm), x read directly.
+// so more CTAs per SM), then read with direct loads; 3: the metric tile in shared memory or on its way
+// there (staged by the caller for several right-hand sides, gsm; gbar != nullptr: the copy completes
+// phase gphase of *gbar, waited for before the physics step), x read directly.
 // Line buffers of metric_tile: three for 4-byte elements; two for 8-byte ones (double-float and FP64
 // arithmetic), whose y-derivatives go back into buffer 0 after one more barrier: with the metric staged
 // a CTA then needs 72 instead of 80 bytes of shared memory per value (K+M), which is one more CTA per SM
@@ -405,10 +406,10 @@ __host__ __device__ constexpr size_t metric_smem_bytes(int nc, int stage)
 // reaches memory.
 // An expired wait for a staged copy: record it in the device status word and wait once more (bounded)
 // so that the copy is not left in flight. Out of line: the common path carries none of it.
-static __device__ __noinline__ void wait_expired(unsigned *status, uint64_t *bar, uint32_t lim)
+static __device__ __noinline__ void wait_expired(unsigned *status, uint64_t *bar, uint32_t lim, uint32_t phase = 0)
 {
     if (status) atomicOr(status, kDevStatusTimeout);
-    mbar_wait_bounded(bar, 0, lim);
+    mbar_wait_bounded(bar, phase, lim);
 }
 
 // Staged tiles and their waits: every wait for a bulk copy is bounded. A thread whose wait expired
@@ -427,7 +428,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                                             int64_t tile, int cpt, unsigned char *smem_raw, df64 *dot = nullptr,
                                             int asm_nx = 0, const VS *sb = nullptr, const VS *sd = nullptr,
                                             unsigned *status = nullptr, uint32_t dbg_extra = 0,
-                                            const GS *gsm = nullptr)
+                                            const GS *gsm = nullptr, uint64_t *gbar = nullptr, uint32_t gphase = 0)
 {
     static_assert(!(RC && STAGE == 1), "recomputed geometry has no metric tile to stage");
     // Double-float renormalisation of the intermediate values: kept where the operator serves the
@@ -605,6 +606,11 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
             if (g_smem) {
                 g_ok = mbar_wait_bounded(bar + 1, 0, lim);
                 if (!g_ok) wait_expired(status, bar + 1, lim);
+            }
+        } else if constexpr (STAGE == 3) {
+            if (gbar) {  // block-uniform
+                g_ok = mbar_wait_bounded(gbar, gphase, lim);
+                if (!g_ok) wait_expired(status, gbar, lim, gphase);
             }
         }
         // (4) quadrature-point physics on the owned pencil, qp = (ra, rb, k)

@@ -31,6 +31,7 @@ struct Batch {
     const Tables1D *tabs[9] = {nullptr};
     size_t smem = 0;
     int grid = 0;
+    int sms = 1;
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph = nullptr;
     // grouped mode: the degree groups run on their own streams, forked from and joined to the
@@ -66,6 +67,16 @@ static cw_status batch_rebuild(Batch &b)
         b.g_first[n] = b.g_count[n] = b.g_items[n] = 0;
         b.g_kind[n] = 0;
     }
+    auto tile_of = [&](int n) {  // cells per tile
+        return b.mode == CW_BATCH_SINGLE ? batch_cpt(n, b.half[n]) : degree_cpb(n, b.variant[n] & 1, !b.fp64);
+    };
+    auto carries_all_rhs = [&](int n) { return b.mode == CW_BATCH_GROUPED && (b.variant[n] >> 1) == 1; };
+    int64_t tiles[9] = {0};  // tiles (times right-hand sides unless an item carries them all) per launch: [0] or [n]
+    for (size_t i = 0; i < b.ops.size(); ++i) {
+        const Op &o = *b.ops[i];
+        const int64_t t = (o.E + tile_of(o.n) - 1) / tile_of(o.n);
+        tiles[b.mode == CW_BATCH_SINGLE ? 0 : o.n] += t * (carries_all_rhs(o.n) ? 1 : b.nrhs[i]);
+    }
     for (size_t i = 0; i < b.ops.size(); ++i) {
         const Op &o = *b.ops[i];
         BatchProb &P = b.h_probs[i];
@@ -78,13 +89,13 @@ static cw_status batch_rebuild(Batch &b)
         P.n = o.n;
         P.kind = o.kind;
         P.nrhs = b.nrhs[i];
-        P.cpt = b.mode == CW_BATCH_SINGLE ? batch_cpt(o.n, b.half[o.n]) : degree_cpb(o.n, b.variant[o.n] & 1, !b.fp64);
+        P.cpt = tile_of(o.n);
         P.ntiles = (o.E + P.cpt - 1) / P.cpt;
         // grouped items with the metric staged once (staging mode 1) carry every right-hand side of
         // their tiles: fewer tiles per item
-        const bool all_rhs = b.mode == CW_BATCH_GROUPED && (b.variant[o.n] >> 1) == 1;
+        const bool all_rhs = carries_all_rhs(o.n);
         const int rh = all_rhs ? P.nrhs : 1;
-        P.tpi = std::max(1, kItemValues / (P.cpt * o.n * o.n * o.n * rh));
+        P.tpi = item_tiles(tiles[b.mode == CW_BATCH_SINGLE ? 0 : o.n], P.cpt * o.n * o.n * o.n * rh, b.sms);
         if (b.mode == CW_BATCH_GROUPED && b.g_count[o.n] == 0) {  // items restart per degree group
             b.g_first[o.n] = (int64_t)i;
             item = 0;
@@ -100,12 +111,10 @@ static cw_status batch_rebuild(Batch &b)
     b.nitems = item;
     b.smem = smem;
     if (b.mode == CW_BATCH_SINGLE) {
-        int per_sm = 0, dev = 0, sms = 0;
+        int per_sm = 0;
         CW_CUDA_TRY(b.fp64 ? batch_occupancy_df(smem, &per_sm) : batch_occupancy_f32(smem, &per_sm));
-        CW_CUDA_TRY(cudaGetDevice(&dev));
-        CW_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         if (per_sm < 1) return fail(CW_ERR_UNSUPPORTED, "cw_batch: kernel does not fit on an SM");
-        b.grid = sms * per_sm;
+        b.grid = b.sms * per_sm;
     }
     // the table is rewritten in place: a launch still running on a non-blocking stream, which a
     // synchronous copy does not wait for, may be reading it
@@ -194,7 +203,14 @@ cw_status cw_batch_create(const cw_op *ops, const int *nrhs, const void *const *
         tabs[o->n] = &o->tab;
         b->tabs[o->n] = &o->tab;
     }
-    cudaError_t e = b->fp64 ? batch_upload_tables_df(tabs) : batch_upload_tables_f32(tabs);
+    // default variants: the per-operator kernel's default tile and staging (in FP32 staging mode 1 with
+    // the metric of a tile staged once for all right-hand sides)
+    for (int n = 2; n <= 8; ++n)
+        b->variant[n] = 2 * default_stage(n, !b->fp64) + (default_cells(n, !b->fp64, true) ? 1 : 0);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = b->fp64 ? batch_upload_tables_df(tabs) : batch_upload_tables_f32(tabs);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_probs, nprob * sizeof(BatchProb));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, 9 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);

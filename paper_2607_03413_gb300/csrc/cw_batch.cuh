@@ -21,7 +21,18 @@
 namespace cw {
 
 constexpr int kBatchThreads = 128;
-constexpr int kItemValues = 16384;  // target cell-wise values per work item
+constexpr int kItemValues = 16384;  // most cell-wise values per work item
+// Tiles per work item of a group of problems with `tiles` tiles (times right-hand sides, where an item
+// carries one): items of about kItemValues values where there are many, but at least kItemsPerSm items
+// per SM, so that the persistent CTAs stay busy to the end. With items of 16384 values throughout, small
+// groups had fewer items than the SMs have CTA slots (15 items of the Q3 problems of an 8 RHS + 12 problem
+// batch: 176 us on 15 SMs).
+constexpr int kItemsPerSm = 24;
+inline int item_tiles(int64_t tiles, int tile_values, int sms)
+{
+    const int64_t most = kItemValues / tile_values, want = tiles / ((int64_t)kItemsPerSm * sms);
+    return (int)(want < 1 || most < 1 ? 1 : want < most ? want : most);
+}
 
 // cells per tile of degree N (n = N nodes): full or half
 __host__ __device__ constexpr int batch_cpt(int N, int half)
@@ -66,6 +77,24 @@ __device__ __forceinline__ const TabMetric<N, C> &batch_tab(const BatchTables<C>
     else return T.t8;
 }
 
+// Called by every thread of a CTA with at least 32 threads: warp 0 takes the number of the CTA's next
+// item and finds the problem of item `it` (the last one whose first item is <= it), 32 table entries at
+// a time: one load instead of a serial chain of log2(nprob) dependent ones.
+__device__ __forceinline__ void next_item(const BatchProb *__restrict__ probs, int nprob, long long it,
+                                          unsigned long long *__restrict__ counter, long long *s_next, int *s_prob)
+{
+    if (threadIdx.x >= 32) return;
+    if (threadIdx.x == 0) *s_next = static_cast<long long>(atomicAdd(counter, 1ull));  // used after this item
+    int cnt = 0;
+    for (int base = 0; base < nprob; base += 32) {
+        const int i = base + static_cast<int>(threadIdx.x);
+        const unsigned m = __ballot_sync(0xffffffffu, i < nprob && __ldg(&probs[i].item0) <= it);
+        cnt += __popc(m);
+        if (m != 0xffffffffu) break;
+    }
+    if (threadIdx.x == 0) *s_prob = cnt - 1;
+}
+
 // one work item of degree N; kept out of line so that each degree gets its own register allocation
 // (all seven bodies inlined into one function spill heavily)
 template <class Ar, class VS, class GS, int N>
@@ -99,16 +128,7 @@ __device__ __forceinline__ void batch_body(const BatchProb *__restrict__ probs, 
         const long long it = s_next;
         if (it >= nitems) return;  // block-uniform
         __syncthreads();           // every thread has read s_next
-        if (threadIdx.x == 0) {
-            s_next = static_cast<long long>(atomicAdd(counter, 1ull));  // next item, used after this one
-            int lo = 0, hi = nprob - 1;
-            while (lo < hi) {  // last problem whose first item is <= it
-                const int mid = (lo + hi + 1) / 2;
-                if (__ldg(&probs[mid].item0) <= it) lo = mid;
-                else hi = mid - 1;
-            }
-            s_prob = lo;
-        }
+        next_item(probs, nprob, it, counter, &s_next, &s_prob);
         __syncthreads();
         const BatchProb P = probs[s_prob];
         const int64_t local = it - P.item0;
@@ -135,22 +155,24 @@ __device__ __forceinline__ const BatchTables<C> &batch_tables();
 // the call costs them more than it saves.) gsm: the tile's metric in shared memory (STAGE 3).
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
 __device__ __noinline__ void grouped_tile(const VS *x, VS *y, const GS *g, int64_t ncells, int kind, int64_t tile,
-                                          unsigned *status, const GS *gsm)
+                                          unsigned *status, const GS *gsm, uint64_t *gbar, uint32_t gphase)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     metric_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, batch_tab<N>(batch_tables<typename Ar::C>()), tile,
-                                           CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm);
+                                           CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gbar, gphase);
 }
 
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
 __device__ __forceinline__ void grouped_one(const VS *x, VS *y, const GS *g, int64_t ncells, int kind, int64_t tile,
-                                            unsigned *status, const GS *gsm, unsigned char *smem_raw)
+                                            unsigned *status, const GS *gsm, uint64_t *gbar, uint32_t gphase,
+                                            unsigned char *smem_raw)
 {
     if constexpr (std::is_same<Ar, ArDF>::value)
-        grouped_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, gsm);
+        grouped_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, gsm, gbar, gphase);
     else
         metric_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, batch_tab<N>(batch_tables<typename Ar::C>()),
-                                               tile, CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm);
+                                               tile, CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gbar,
+                                               gphase);
 }
 
 // ---- grouped mode: one persistent kernel per degree, shaped like the per-operator kernel
@@ -173,22 +195,17 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
     const size_t offb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), true>::RS * sizeof(T);  // a multiple of 16
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + offb);
     GS *sG = reinterpret_cast<GS *>(smem_raw + offb + 16);
-    if (threadIdx.x == 0) s_next = static_cast<long long>(atomicAdd(counter, 1ull));
+    [[maybe_unused]] uint32_t phase = 0;  // of the metric tile's barrier
+    if (threadIdx.x == 0) {
+        if constexpr (STAGE == 1) mbar_init(bar, 1);
+        s_next = static_cast<long long>(atomicAdd(counter, 1ull));
+    }
     for (;;) {
         __syncthreads();
         const long long it = s_next;
         if (it >= nitems) return;  // block-uniform
         __syncthreads();
-        if (threadIdx.x == 0) {
-            s_next = static_cast<long long>(atomicAdd(counter, 1ull));
-            int lo = 0, hi = nprob - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) / 2;
-                if (__ldg(&probs[mid].item0) <= it) lo = mid;
-                else hi = mid - 1;
-            }
-            s_prob = lo;
-        }
+        next_item(probs, nprob, it, counter, &s_next, &s_prob);
         __syncthreads();
         const BatchProb P = probs[s_prob];
         const int64_t local = it - P.item0;
@@ -208,19 +225,9 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
                 const GS *gsrc = g + cell0 * NC * N3;
                 const uint32_t gb = CPB * NC * N3 * sizeof(GS);
                 staged = cell0 + CPB <= P.ncells && aligned16(gsrc) && gb % 16 == 0;  // block-uniform
-                if (staged) {
-                    if (threadIdx.x == 0) mbar_init(bar, 1);
-                    __syncthreads();
-                    if (threadIdx.x == 0) {
-                        mbar_expect_tx(bar, gb);
-                        bulk_g2s(sG, gsrc, gb, bar);
-                    }
-                    const bool ok = mbar_wait_bounded(bar, 0, kWaitLimit);
-                    if (!ok) {  // reported; the copy is waited for once more, the tile reads from global memory
-                        if (P.status) atomicOr(P.status, kDevStatusTimeout);
-                        mbar_wait_bounded(bar, 0, kWaitLimit);
-                    }
-                    staged = !__syncthreads_or(!ok);
+                if (staged && threadIdx.x == 0) {  // waited for before the first right-hand side's physics
+                    mbar_expect_tx(bar, gb);
+                    bulk_g2s(sG, gsrc, gb, bar);
                 }
             }
             for (int r = r0; r < r1; ++r) {
@@ -229,11 +236,14 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
                 VS *y = static_cast<VS *>(P.y) + r * P.stride;
                 if constexpr (STAGE == 1) {  // one code path: the metric from shared or from global memory
                     const GS *gm = staged ? sG : g + tile * CPB * NC * N3;
-                    grouped_one<N, CPB, Ar, VS, GS, 3>(x, y, g, P.ncells, P.kind, tile, P.status, gm, smem_raw);
+                    grouped_one<N, CPB, Ar, VS, GS, 3>(x, y, g, P.ncells, P.kind, tile, P.status, gm,
+                                                       staged && r == r0 ? bar : nullptr, phase, smem_raw);
                 } else {
-                    grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status, nullptr, smem_raw);
+                    grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status, nullptr, nullptr,
+                                                           0, smem_raw);
                 }
             }
+            if (staged) phase ^= 1u;
         }
     }
 }
