@@ -367,6 +367,126 @@ __global__ void dss_xtile_kernel(VS *__restrict__ v, int nx, int p, int xtile, i
 }
 
 
+// All passes of Algorithm struct_dss in one launch, for one or several structured meshes whose vectors
+// are parts of one array (the blocks of a multi-block mesh). One thread per node of the continuous grid: a
+// node on interior cell faces has 2, 4 or 8 copies, which its thread reads, sums in the passes' order (x
+// pairs, then y, then z; HALF: each sum halved) and writes back, so the sum is in place and bit-identical to
+// the passes. Nodes inside cells leave at once. x-interfaces whose right
+// cell K has K & xmask != 0 (all of them for xmask = -1) were summed already: both copies hold the sum.
+// (One thread per cell-wise entry, the lowest copy of a node working, kept 30 % of the lanes busy at p = 3
+// and took 25 us for 10^6 FP64 values.)
+struct DssMesh {
+    int64_t off;     // first entry of the mesh's vector
+    uint32_t cta0;   // first CTA that works on it
+    uint32_t nodes;  // (nx p + 1)(ny p + 1)(nz p + 1)
+    int nx, ny, nz, xmask;
+    FastDiv fgx, fgy;  // by nx p + 1, ny p + 1
+};
+constexpr int kDssMeshes = 16;  // meshes per launch (the table is a kernel parameter)
+struct DssMeshes {
+    DssMesh m[kDssMeshes];
+    int count;
+};
+
+// s / 2 (exact but for subnormal results), in FP64 by the exponent field: a multiply would occupy the slow
+// FP64 pipe
+template <class VS>
+__device__ __forceinline__ VS half_of(VS s) { return MulOp<VS>::mul(s, 0.5); }
+template <>
+__device__ __forceinline__ double half_of<double>(double s)
+{
+    const int hi = __double2hiint(s), e = hi & 0x7ff00000;
+    if (e <= 0x00100000 || e == 0x7ff00000) return s * 0.5;  // zero, results below the normal range, inf, NaN
+    return __hiloint2double(hi - 0x00100000, __double2loint(s));
+}
+
+template <class VS, bool HALF>
+__global__ void __launch_bounds__(256) dss_node_kernel(VS *__restrict__ v0, int p, FastDiv fp,
+                                                       const __grid_constant__ DssMeshes tab)
+{
+    int b = 0;
+    while (b + 1 < tab.count && tab.m[b + 1].cta0 <= blockIdx.x) ++b;
+    const uint32_t t = (blockIdx.x - tab.m[b].cta0) * 256u + threadIdx.x;
+    if (t >= tab.m[b].nodes) return;
+    const int n = p + 1, nx = tab.m[b].nx, ny = tab.m[b].ny, nz = tab.m[b].nz;
+    const uint32_t line = tab.m[b].fgx.div(t), gz = tab.m[b].fgy.div(line);
+    const uint32_t g[3] = {t - line * tab.m[b].fgx.d, line - gz * tab.m[b].fgy.d, gz};
+    const int nc[3] = {nx, ny, nz};
+    int c[3], l[3];  // cell and local index of the node's lowest copy
+    bool h[3];       // on an interior interface normal to the axis
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        c[a] = static_cast<int>(fp.div(g[a]));
+        l[a] = static_cast<int>(g[a]) - c[a] * p;
+        h[a] = l[a] == 0 && c[a] > 0 && c[a] < nc[a];
+        if (l[a] == 0 && c[a] > 0) c[a] -= 1, l[a] = p;
+    }
+    if (!(h[0] || h[1] || h[2])) return;
+    const int64_t n3 = n * n * n, dx = n3 - p, dy = n3 * nx - n * p, dz = n3 * nx * ny - n * n * p;
+    const uint32_t K = c[0] + nx * (c[1] + ny * c[2]);
+    VS *v = v0 + tab.m[b].off + K * n3 + l[0] + n * (l[1] + n * l[2]);
+    const uint32_t xmask = static_cast<uint32_t>(tab.m[b].xmask);
+    auto pair = [](VS l, VS r) {
+        const VS s = AddOp<VS>::add(l, r);
+        if constexpr (HALF) return half_of(s);
+        else return s;
+    };
+    auto xsum = [&](int64_t o, uint32_t Kl) {  // x pass at one (y, z) copy whose left cell is Kl
+        return h[0] && ((Kl + 1) & xmask) == 0 ? pair(v[o], v[o + dx]) : v[o];
+    };
+    auto ysum = [&](int64_t o, uint32_t Kl) {
+        const VS s = xsum(o, Kl);
+        return h[1] ? pair(s, xsum(o + dy, Kl + nx)) : s;
+    };
+    VS s = ysum(0, K);
+    if (h[2]) s = pair(s, ysum(dz, K + nx * ny));
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const bool bx = q & 1, by = q & 2, bz = q & 4;
+        if ((bx && !h[0]) || (by && !h[1]) || (bz && !h[2])) continue;
+        v[(bx ? dx : 0) + (by ? dy : 0) + (bz ? dz : 0)] = s;
+    }
+}
+
+// Where the one launch is used, by measurement (us per DSS in a CUDA graph, one launch / passes, with 1e5,
+// 3e5, 1e6 and 8e6 entries): Q3 FP64 4.2/5.7, 5.4/6.5, 9.1/10, 44/43; Q4 FP64 4.4/5.8, 5.9/6.6, 11/9.1,
+// 51/41; Q3 FP32 3.6/5.3, 5.4/5.7, 9.7/8.1, 44/29; Q7 FP32 3.4/5.2, 4.4/5.3, 7.0/6.8, 33/21; but Q1, where
+// every node is shared, 3.9/5.5, 4.3/7.3, 9.2/12, 45/60 in FP64 and 3.2/5.4, 3.7/6.3, 6.6/10, 31/50 in
+// FP32. So: at Q1 always, else up to 2^19 entries, and up to 2^21 entries per block where it also saves the
+// launches of several blocks.
+static bool dss_one_launch(const Op &op, int meshes)
+{
+    if (op.L >= ((int64_t)1 << 31) - (1 << 20)) return false;  // 32-bit node and cell numbers
+    return op.p == 1 || op.L <= ((int64_t)1 << (meshes > 1 ? 21 : 19));
+}
+
+// one launch for `count` <= kDssMeshes meshes of one degree; xtile[b] as in dss_launch (0: none, -1: all)
+template <class VS>
+static cudaError_t dss_node_typed(const Op *const *ops, const int64_t *off, const int *xtile, int count, VS *v,
+                                  int flags, cudaStream_t s)
+{
+    DssMeshes tab;
+    uint32_t cta = 0;
+    for (int b = 0; b < count; ++b) {
+        const Mesh &m = *ops[b]->mesh;
+        DssMesh &d = tab.m[b];
+        d.off = off ? off[b] : 0;
+        d.cta0 = cta;
+        d.nodes = (uint32_t)(((int64_t)m.nx * ops[b]->p + 1) * ((int64_t)m.ny * ops[b]->p + 1) * ((int64_t)m.nz * ops[b]->p + 1));
+        d.nx = m.nx, d.ny = m.ny, d.nz = m.nz;
+        d.xmask = xtile[b] < 0 ? -1 : xtile[b] > 1 ? xtile[b] - 1 : 0;  // tiles hold a power of two of cells
+        d.fgx = FastDiv::make(m.nx * ops[b]->p + 1);
+        d.fgy = FastDiv::make(m.ny * ops[b]->p + 1);
+        cta += (d.nodes + 255) / 256;
+    }
+    tab.count = count;
+    const int p = ops[0]->p;
+    const FastDiv fp = FastDiv::make(p);
+    if (flags == CW_DSS_AVERAGE) dss_node_kernel<VS, true><<<cta, 256, 0, s>>>(v, p, fp, tab);
+    else dss_node_kernel<VS, false><<<cta, 256, 0, s>>>(v, p, fp, tab);
+    return cudaGetLastError();
+}
+
 // dst = src with the x pass of Algorithm struct_dss applied: an entry on an interior x-face adds its
 // partner copy in the neighbouring cell, every other entry is copied (out of place, so the read of
 // a partner never sees an updated value). Replaces a copy and an in-place x pass with one pass.
@@ -516,6 +636,11 @@ static cudaError_t dss_typed(const Op &op, VS *v, int flags, cudaStream_t s, int
     const Mesh &m = *op.mesh;
     const int dims[3] = {m.nx, m.ny, m.nz};
     const int n2 = op.n * op.n;
+    if (first_axis <= 1 && end_axis == 3 && dss_one_launch(op, 1)) {
+        const Op *o = &op;
+        const int xt = first_axis == 1 ? -1 : xtile;
+        return dss_node_typed(&o, nullptr, &xt, 1, v, flags, s);
+    }
     for (int ax = first_axis; ax < end_axis; ++ax) {
         if (dims[ax] < 2) continue;
         // in-face coordinates: a = lower of the two other axes (x-index part), b = the other (grid y)
@@ -565,6 +690,27 @@ cudaError_t dss_launch(const Op &op, void *v, int flags, cudaStream_t s, int xti
     }
 }
 
+cudaError_t dss_multi_launch(const Op *const *ops, const int64_t *off, const int *xtile, int count, void *v, int flags,
+                             cudaStream_t s)
+{
+    bool one = true;
+    for (int b = 0; b < count; ++b) one = one && dss_one_launch(*ops[b], count);
+    const size_t es = vec_elem_size(ops[0]->prec);
+    for (int b = 0; b < count;) {
+        const int c = one ? std::min(count - b, kDssMeshes) : 1;
+        void *vb = static_cast<char *>(v) + off[b] * es;
+        cudaError_t e;
+        if (!one)
+            e = flags == CW_DSS_AVERAGE ? dss_average_launch(*ops[b], vb, s, xtile[b]) : dss_launch(*ops[b], vb, flags, s, xtile[b]);
+        else if (es == 8) e = dss_node_typed(ops + b, off + b, xtile + b, c, static_cast<double *>(v), flags, s);
+        else if (es == 4) e = dss_node_typed(ops + b, off + b, xtile + b, c, static_cast<float *>(v), flags, s);
+        else e = dss_node_typed(ops + b, off + b, xtile + b, c, static_cast<__nv_bfloat16 *>(v), flags, s);
+        if (e != cudaSuccess) return e;
+        b += c;
+    }
+    return cudaSuccess;
+}
+
 // sum passes of the axes [ax0, ax1) only (no averaging); used on slab views of the mesh
 static cudaError_t dss_axes(const Op &op, void *v, int ax0, int ax1, cudaStream_t s, int xtile = 0)
 {
@@ -582,6 +728,35 @@ cudaError_t apply_local(const Op &op, const void *x, void *y, cudaStream_t s, in
     case CW_PREC_F64_NATIVE: return apply_launch_f64n(op, x, y, s, xfuse);
     default: return apply_launch_f32(op, x, y, s, xfuse);
     }
+}
+
+// One launch per 16 operators where all store their metric and run their default variant; else one per
+// operator.
+cudaError_t apply_multi_launch(const Op *const *ops, const int64_t *off, int count, const void *x, void *y, int *xtile,
+                               cudaStream_t s)
+{
+    const Op &o0 = *ops[0];
+    const bool f32 = o0.prec == CW_PREC_F32;
+    bool one = count > 1 && (f32 || o0.prec == CW_PREC_F64);
+    const int half = tile_cells(o0.n, f32) / 2;
+    int64_t tiles = 0;
+    for (int b = 0; b < count; ++b) {
+        const Op &o = *ops[b];
+        one = one && o.geom == CW_GEOM_METRIC && o.stage == default_stage(o.n, f32) &&
+              o.cpb == (default_cells(o.n, f32, true) ? half : 0);
+        tiles += o.E;
+    }
+    if (one && tiles < ((int64_t)1 << 31))
+        return f32 ? apply_multi_launch_f32(ops, off, count, x, y, xtile, s)
+                   : apply_multi_launch_df(ops, off, count, x, y, xtile, s);
+    const size_t es = vec_elem_size(o0.prec);
+    for (int b = 0; b < count; ++b) {
+        const bool fuse = xtile && ops[b]->E * (int64_t)(o0.n * o0.n) < ((int64_t)1 << 32);
+        cudaError_t e = apply_local(*ops[b], static_cast<const char *>(x) + off[b] * es,
+                                    static_cast<char *>(y) + off[b] * es, s, fuse ? xtile + b : nullptr);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // ----------------------------------------------------------- diagonal and load vector ----

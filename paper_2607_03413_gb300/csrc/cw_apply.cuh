@@ -874,6 +874,36 @@ __global__ void __launch_bounds__(N *N *CPB, (df_min_blocks<N * N * CPB, RC>()))
                                                       asm_nx, nullptr, nullptr, status, dbg_extra);
 }
 
+// Several operators of one degree, kind and precision in one launch (the blocks of a multi-block mesh, each
+// too small to fill the GPU): CTA blockIdx.x works on tile blockIdx.x - tile0 of the last operator of the
+// table with tile0 <= blockIdx.x. x and y are the concatenated vectors.
+struct MultiOp {
+    int64_t off, ncells;
+    const void *geo;
+    unsigned *status;
+    unsigned tile0;
+    int asm_nx;
+    uint32_t dbg_extra;
+};
+constexpr int kMultiOps = 16;  // operators per launch (the table is a kernel parameter)
+struct MultiOps {
+    MultiOp o[kMultiOps];
+    int count;
+};
+template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
+__global__ void __launch_bounds__(N *N *CPB, (df_capped<Ar, N, false>() ? df_min_blocks<N * N * CPB, false>() : 0))
+    apply_multi_kernel(const VS *__restrict__ x, VS *__restrict__ y, int kind, TabMetric<N, typename Ar::C> tab,
+                       const __grid_constant__ MultiOps ops)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int b = 0;
+    while (b + 1 < ops.count && ops.o[b + 1].tile0 <= blockIdx.x) ++b;
+    const MultiOp &o = ops.o[b];
+    metric_tile<N, CPB, Ar, VS, GS, STAGE>(x + o.off, y + o.off, static_cast<const GS *>(o.geo), o.ncells, kind, tab,
+                                           blockIdx.x - o.tile0, CPB, smem_raw, nullptr, o.asm_nx, nullptr, nullptr,
+                                           o.status, o.dbg_extra);
+}
+
 // y = A x and the CTA's partial of <x, A x> in part[blockIdx.x] (deterministic: fixed order in a CTA)
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE, bool RC = false>
 __global__ void __launch_bounds__(N *N *CPB) apply_metric_dot_kernel(const VS *__restrict__ x, VS *__restrict__ y,

@@ -15,4 +15,9 @@ cudaError_t apply_dot_launch_f32(const Op &op, const void *x, void *y, double *p
 {
     return launch_dot_degree<ArF32, float, float>(op, x, y, part, nb, s);
 }
+cudaError_t apply_multi_launch_f32(const Op *const *ops, const int64_t *off, int count, const void *x, void *y,
+                                   int *xtile, cudaStream_t s)
+{
+    return launch_multi_degree<ArF32, float, float>(ops, off, count, x, y, xtile, s);
+}
 }  // namespace cw

@@ -128,6 +128,18 @@ cudaError_t apply_dot_launch_f32g16(const Op &op, const void *x, void *y, double
 cudaError_t apply_local(const Op &op, const void *x, void *y, cudaStream_t s, int *xfuse = nullptr);
 // xtile > 0: the x pass skips the interfaces inside tiles of xtile consecutive cells (already summed)
 cudaError_t dss_launch(const Op &op, void *v, int flags, cudaStream_t s, int xtile = 0);
+// the same on `count` meshes of one degree and vector type whose vectors start at off[b] of v (one launch
+// for up to 16 small meshes)
+cudaError_t dss_multi_launch(const Op *const *ops, const int64_t *off, const int *xtile, int count, void *v, int flags,
+                             cudaStream_t s);
+// y = A x on `count` operators of one degree, kind and precision whose vectors start at off[b] of x and y,
+// in as few launches as possible; xtile (may be NULL): as xfuse of apply_local, one entry per operator
+cudaError_t apply_multi_launch(const Op *const *ops, const int64_t *off, int count, const void *x, void *y, int *xtile,
+                               cudaStream_t s);
+cudaError_t apply_multi_launch_df(const Op *const *ops, const int64_t *off, int count, const void *x, void *y,
+                                  int *xtile, cudaStream_t s);
+cudaError_t apply_multi_launch_f32(const Op *const *ops, const int64_t *off, int count, const void *x, void *y,
+                                   int *xtile, cudaStream_t s);
 // out of place: dst = S src (flags CW_DSS_SUM) or S_bar src (CW_DSS_AVERAGE); the x pass is fused
 // with the copy
 cudaError_t dss_from(const Op &op, const void *src, void *dst, int flags, cudaStream_t s);

@@ -199,6 +199,50 @@ cudaError_t launch_metric(const Op &op, const void *x, void *y, cudaStream_t s, 
     return cudaGetLastError();
 }
 
+// several stored-metric operators in their default variant, at most kMultiOps per launch
+template <int N, class Ar, class VS, class GS>
+cudaError_t launch_multi(const Op *const *op, const int64_t *off, int count, const void *x, void *y, int *xtile,
+                         cudaStream_t s)
+{
+    constexpr int CPB = cpb_tuned<N, Ar, VS>(), ST = default_stage(N, std::is_same<Ar, ArF32>::value);
+    TabMetric<N, typename Ar::C> tab;
+    fill_metric_tab<N>(tab, op[0]->tab, [](double v) { return MakeC<Ar>::from(v); });
+    const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op[0]->kind), ST);
+    auto kern = apply_multi_kernel<N, CPB, Ar, VS, GS, ST>;
+    static size_t opted[kMaxDevices] = {};
+    if (cudaError_t e = ensure_smem(kern, smem, opted); e != cudaSuccess) return e;
+    for (int b0 = 0; b0 < count; b0 += kMultiOps) {
+        MultiOps t;
+        t.count = std::min(kMultiOps, count - b0);
+        unsigned tiles = 0;
+        for (int b = 0; b < t.count; ++b) {
+            const Op &o = *op[b0 + b];
+            t.o[b] = MultiOp{off[b0 + b], o.E, o.d_geo, o.d_status, tiles, xtile ? o.mesh->nx : 0, o.dbg_tma_extra};
+            tiles += (unsigned)((o.E + CPB - 1) / CPB);
+            if (xtile) xtile[b0 + b] = CPB;
+        }
+        kern<<<tiles, N * N * CPB, smem, s>>>(static_cast<const VS *>(x), static_cast<VS *>(y), op[0]->kind, tab, t);
+        if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+template <class Ar, class VS, class GS>
+cudaError_t launch_multi_degree(const Op *const *op, const int64_t *off, int count, const void *x, void *y, int *xtile,
+                                cudaStream_t s)
+{
+    switch (op[0]->n) {
+    case 2: return launch_multi<2, Ar, VS, GS>(op, off, count, x, y, xtile, s);
+    case 3: return launch_multi<3, Ar, VS, GS>(op, off, count, x, y, xtile, s);
+    case 4: return launch_multi<4, Ar, VS, GS>(op, off, count, x, y, xtile, s);
+    case 5: return launch_multi<5, Ar, VS, GS>(op, off, count, x, y, xtile, s);
+    case 6: return launch_multi<6, Ar, VS, GS>(op, off, count, x, y, xtile, s);
+    case 7: return launch_multi<7, Ar, VS, GS>(op, off, count, x, y, xtile, s);
+    case 8: return launch_multi<8, Ar, VS, GS>(op, off, count, x, y, xtile, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
 // One fused smoothing sweep (smooth_metric_kernel): default tile, input tile staged by TMA and, where
 // the metric is stored, the arithmetic's default staging of it (FP32: prefetched into L2); the x-interfaces inside tiles are averaged, *xfuse receives the
 // tile size for the x pass between tiles.

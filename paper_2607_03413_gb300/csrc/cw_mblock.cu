@@ -35,7 +35,8 @@ namespace cw {
 
 // ------------------------------------------------------------------------------ kernels ----
 // One entity per thread: s = sum of its representatives (one copy per sharing block, in block order),
-// then s to every copy. Entities touch disjoint copies, so the launch needs no atomics.
+// then s to every copy. Entities touch disjoint copies, also across the codimension sets, so one launch
+// over the three sets needs no atomics.
 template <class VS>
 struct MbAcc {
     using A = VS;
@@ -49,13 +50,24 @@ struct MbAcc<__nv_bfloat16> {
     static __device__ __forceinline__ __nv_bfloat16 to(float a) { return __float2bfloat16_rn(a); }
 };
 
+struct MbSet {  // one codimension set of shared DoFs, CSR tables on the device
+    int64_t nent = 0;
+    int64_t *rptr = nullptr, *rep = nullptr, *cptr = nullptr, *cp = nullptr;
+};
+
+struct MbSets {
+    MbSet s[3];
+};
+
 template <class VS>
-__global__ void mb_entity_kernel(VS *__restrict__ v, int64_t nent, const int64_t *__restrict__ rptr,
-                                 const int64_t *__restrict__ rep, const int64_t *__restrict__ cptr,
-                                 const int64_t *__restrict__ cp)
+__global__ void mb_entity_kernel(VS *__restrict__ v, const __grid_constant__ MbSets sets)
 {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nent) return;
+    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int k = 0;
+    while (k < 2 && e >= sets.s[k].nent) e -= sets.s[k++].nent;
+    if (e >= sets.s[k].nent) return;
+    const int64_t *__restrict__ rptr = sets.s[k].rptr, *__restrict__ rep = sets.s[k].rep;
+    const int64_t *__restrict__ cptr = sets.s[k].cptr, *__restrict__ cp = sets.s[k].cp;
     typename MbAcc<VS>::A s = MbAcc<VS>::from(v[rep[rptr[e]]]);
     for (int64_t r = rptr[e] + 1; r < rptr[e + 1]; ++r) s = s + MbAcc<VS>::from(v[rep[r]]);
     const VS o = MbAcc<VS>::to(s);
@@ -73,17 +85,13 @@ __global__ void mb_divide_kernel(VS *__restrict__ v, const uint8_t *__restrict__
 }
 
 // ---------------------------------------------------------------------------- structure ----
-struct MbSet {  // one codimension set of shared DoFs, CSR tables on the device
-    int64_t nent = 0;
-    int64_t *rptr = nullptr, *rep = nullptr, *cptr = nullptr, *cp = nullptr;
-};
-
 struct MBlock {
     std::vector<Op *> ops;
     std::vector<int64_t> off;  // first cell-wise entry of every block; off.back() = L
     int p = 0, n = 0, prec = 0;
     int64_t L = 0, NG = 0;
-    MbSet sets[3];             // macro-face interiors, macro-line interiors, macro-vertices
+    MbSets all;
+    MbSet (&sets)[3] = all.s;  // macro-face interiors, macro-line interiors, macro-vertices
     uint8_t *kappa = nullptr;  // number of copies of every entry's DoF
     uint8_t *dirichlet = nullptr;  // 1 on entries of DoFs on the domain boundary (unglued block faces)
     std::vector<int64_t> gidx; // global DoF of every entry (host)
@@ -388,39 +396,39 @@ static cw_status mblock_build(MBlock &mb)
 }
 
 template <class VS>
-static cudaError_t mb_dss_typed(const MBlock &mb, VS *v, int flags, cudaStream_t s)
+static cudaError_t mb_entities(const MBlock &mb, VS *v, cudaStream_t s)  // Algorithm unstruct_dss
 {
-    for (size_t b = 0; b < mb.ops.size(); ++b) {  // Algorithm struct_dss inside every block
-        cudaError_t e = dss_launch(*mb.ops[b], v + mb.off[b], CW_DSS_SUM, s);
-        if (e != cudaSuccess) return e;
-    }
-    for (const MbSet &S : mb.sets)  // Algorithm unstruct_dss: faces, lines, vertices
-        if (S.nent > 0)
-            mb_entity_kernel<VS><<<(unsigned)((S.nent + 255) / 256), 256, 0, s>>>(v, S.nent, S.rptr, S.rep, S.cptr,
-                                                                                   S.cp);
+    const int64_t nent = mb.sets[0].nent + mb.sets[1].nent + mb.sets[2].nent;
+    if (nent > 0) mb_entity_kernel<VS><<<(unsigned)((nent + 255) / 256), 256, 0, s>>>(v, mb.all);
+    return cudaGetLastError();
+}
+
+// xtile (may be NULL): per block, the tile inside which the operator summed the x-interfaces already
+template <class VS>
+static cudaError_t mb_dss_typed(const MBlock &mb, VS *v, int flags, const int *xtile, cudaStream_t s)
+{
+    const std::vector<int> none(mb.ops.size(), 0);
+    cudaError_t e = dss_multi_launch(mb.ops.data(), mb.off.data(), xtile ? xtile : none.data(), (int)mb.ops.size(), v,
+                                     CW_DSS_SUM, s);  // Algorithm struct_dss inside every block
+    if (e == cudaSuccess) e = mb_entities(mb, v, s);
+    if (e != cudaSuccess) return e;
     if (flags == CW_DSS_AVERAGE)
         mb_divide_kernel<VS><<<1216, 256, 0, s>>>(v, mb.kappa, mb.L);
     return cudaGetLastError();
 }
 
-static cudaError_t mb_dss(const MBlock &mb, void *v, int flags, cudaStream_t s)
+static cudaError_t mb_dss(const MBlock &mb, void *v, int flags, cudaStream_t s, const int *xtile = nullptr)
 {
     switch (vec_elem_size(mb.prec)) {
-    case 8: return mb_dss_typed(mb, static_cast<double *>(v), flags, s);
-    case 4: return mb_dss_typed(mb, static_cast<float *>(v), flags, s);
-    default: return mb_dss_typed(mb, static_cast<__nv_bfloat16 *>(v), flags, s);
+    case 8: return mb_dss_typed(mb, static_cast<double *>(v), flags, xtile, s);
+    case 4: return mb_dss_typed(mb, static_cast<float *>(v), flags, xtile, s);
+    default: return mb_dss_typed(mb, static_cast<__nv_bfloat16 *>(v), flags, xtile, s);
     }
 }
 
-static cudaError_t mb_apply_local(const MBlock &mb, const void *x, void *y, cudaStream_t s)
+static cudaError_t mb_apply_local(const MBlock &mb, const void *x, void *y, cudaStream_t s, int *xtile = nullptr)
 {
-    const size_t es = vec_elem_size(mb.prec);
-    for (size_t b = 0; b < mb.ops.size(); ++b) {
-        cudaError_t e = apply_local(*mb.ops[b], static_cast<const char *>(x) + mb.off[b] * es,
-                                    static_cast<char *>(y) + mb.off[b] * es, s);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return apply_multi_launch(mb.ops.data(), mb.off.data(), (int)mb.ops.size(), x, y, xtile, s);
 }
 
 // ------------------------------------------------------------------ Jacobi-PCG (FP64) ----
@@ -626,8 +634,9 @@ cw_status cw_mblock_apply(cw_mblock h, const void *x, void *y, int flags, void *
     if (flags != CW_APPLY_LOCAL && flags != CW_APPLY_ASSEMBLE) return fail(CW_ERR_ARG, "cw_mblock_apply: bad flags");
     if (x == y) return fail(CW_ERR_ARG, "cw_mblock_apply: x and y must not alias");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    CW_CUDA_TRY(mb_apply_local(*mb, x, y, s));
-    if (flags == CW_APPLY_ASSEMBLE) CW_CUDA_TRY(mb_dss(*mb, y, CW_DSS_SUM, s));
+    std::vector<int> xtile(mb->ops.size(), 0);
+    CW_CUDA_TRY(mb_apply_local(*mb, x, y, s, flags == CW_APPLY_ASSEMBLE ? xtile.data() : nullptr));
+    if (flags == CW_APPLY_ASSEMBLE) CW_CUDA_TRY(mb_dss(*mb, y, CW_DSS_SUM, s, xtile.data()));
     return CW_OK;
 }
 
@@ -640,11 +649,7 @@ cw_status cw_mblock_diagonal(cw_mblock h, double *d, void *stream)
         cw_status st = cw_diagonal(reinterpret_cast<cw_op>(mb->ops[b]), d + mb->off[b], stream);
         if (st != CW_OK) return st;
     }
-    for (const MbSet &S : mb->sets)  // then across the blocks
-        if (S.nent > 0)
-            mb_entity_kernel<double><<<(unsigned)((S.nent + 255) / 256), 256, 0, s>>>(d, S.nent, S.rptr, S.rep, S.cptr,
-                                                                                       S.cp);
-    CW_CUDA_TRY(cudaGetLastError());
+    CW_CUDA_TRY(mb_entities(*mb, d, s));  // then across the blocks
     return CW_OK;
 }
 
