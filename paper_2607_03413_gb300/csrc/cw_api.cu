@@ -17,6 +17,7 @@
 #include "cw_index.cuh"
 #include "cw_internal.h"
 #include "cw_launch.cuh"
+#include "cw_line.cuh"
 
 namespace cw {
 
@@ -490,22 +491,20 @@ static cudaError_t dss_node_typed(const Op *const *ops, const int64_t *off, cons
 // dst = src with the x pass of Algorithm struct_dss applied: an entry on an interior x-face adds its
 // partner copy in the neighbouring cell, every other entry is copied (out of place, so the read of
 // a partner never sees an updated value). Replaces a copy and an in-place x pass with one pass.
-template <class VS, bool HALF = false>
-__global__ void dss_x_from_kernel(const VS *__restrict__ src, VS *__restrict__ dst, int nx, int p, uint32_t nlines,
-                                  FastDiv fd_n2, FastDiv fd_nx)
+template <int N, class VS, bool HALF = false>
+__global__ void dss_x_from_kernel(const VS *__restrict__ src, VS *__restrict__ dst, int nx, uint32_t nlines,
+                                  FastDiv fd_nx)
 {
     // one thread per x-line (n consecutive entries of a cell); only its two end entries have partners
     const uint32_t l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= nlines) return;
-    const int n = p + 1;
-    const uint32_t n3 = fd_n2.d * n;
-    const uint32_t c = fd_n2.div(l);
+    constexpr int n = N, p = N - 1;
+    constexpr uint32_t n3 = N * N * N;
+    const uint32_t c = l / (N * N);
     const uint32_t cx = c - fd_nx.div(c) * static_cast<uint32_t>(nx);
     const int64_t b = static_cast<int64_t>(l) * n;
-    VS v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (i < n) v[i] = src[b + i];
+    VS v[N];
+    line_ld<N>(src + b, v, LineVec<N, VS>::aligned(src));
     if (cx > 0) {
         v[0] = AddOp<VS>::add(src[b - n3 + p], v[0]);
         if constexpr (HALF) v[0] = MulOp<VS>::mul(v[0], 0.5);
@@ -514,9 +513,35 @@ __global__ void dss_x_from_kernel(const VS *__restrict__ src, VS *__restrict__ d
         v[p] = AddOp<VS>::add(v[p], src[b + n3]);
         if constexpr (HALF) v[p] = MulOp<VS>::mul(v[p], 0.5);
     }
+    line_st<N>(dst + b, v, LineVec<N, VS>::aligned(dst));
+}
+
+// a b rounded on its own (not contracted into the sum that follows, so that both copies of a node get the
+// same bits)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// dst = x averages of (d b): the first smoothing sweep from zero (u = D_hat b per copy) with the first pass of
+// the averaging DSS that follows it
+template <int N, class VS>
+__global__ void dss_x_scale_kernel(const VS *__restrict__ b, const VS *__restrict__ d, VS *__restrict__ dst, int nx,
+                                   uint32_t nlines, FastDiv fd_nx)
+{
+    const uint32_t l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l >= nlines) return;
+    constexpr int p = N - 1;
+    constexpr uint32_t n3 = N * N * N;
+    const uint32_t c = l / (N * N);
+    const uint32_t cx = c - fd_nx.div(c) * static_cast<uint32_t>(nx);
+    const int64_t o = static_cast<int64_t>(l) * N;
+    VS v[N], t[N];
+    line_ld<N>(b + o, v, LineVec<N, VS>::aligned(b));
+    line_ld<N>(d + o, t, LineVec<N, VS>::aligned(d));
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (i < n) dst[b + i] = v[i];
+    for (int i = 0; i < N; ++i) v[i] = mul_rn(t[i], v[i]);
+    if (cx > 0) v[0] = half_of(AddOp<VS>::add(mul_rn(d[o - n3 + p], b[o - n3 + p]), v[0]));
+    if (cx + 1 < static_cast<uint32_t>(nx)) v[p] = half_of(AddOp<VS>::add(v[p], mul_rn(d[o + n3], b[o + n3])));
+    line_st<N>(dst + o, v, LineVec<N, VS>::aligned(dst));
 }
 
 // r - a q with one rounding, written once so that every use (own line, partner copy) gives the same value
@@ -527,28 +552,27 @@ __device__ __forceinline__ float resid_update<float>(float r, float q, float a) 
 
 // dst = x pass of (r - a q), a = *active ? *alpha : 0: the CG residual update r <- r - alpha A p fused
 // into the first pass of the DSS that follows it (the updated residual itself is only needed as S r).
-template <class VS>
+template <int N, class VS>
 __global__ void dss_x_axpy_kernel(const VS *__restrict__ r, const VS *__restrict__ q,
                                   const double *__restrict__ alpha, const int *__restrict__ active,
-                                  VS *__restrict__ dst, int nx, int p, uint32_t nlines, FastDiv fd_n2, FastDiv fd_nx)
+                                  VS *__restrict__ dst, int nx, uint32_t nlines, FastDiv fd_nx)
 {
     const uint32_t l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= nlines) return;
     const VS a = *active ? static_cast<VS>(*alpha) : VS(0);
-    const int n = p + 1;
-    const uint32_t n3 = fd_n2.d * n;
-    const uint32_t c = fd_n2.div(l);
+    constexpr int p = N - 1;
+    constexpr uint32_t n3 = N * N * N;
+    const uint32_t c = l / (N * N);
     const uint32_t cx = c - fd_nx.div(c) * static_cast<uint32_t>(nx);
-    const int64_t b = static_cast<int64_t>(l) * n;
-    VS v[8];
+    const int64_t b = static_cast<int64_t>(l) * N;
+    VS v[N], t[N];
+    line_ld<N>(r + b, v, LineVec<N, VS>::aligned(r));
+    line_ld<N>(q + b, t, LineVec<N, VS>::aligned(q));
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (i < n) v[i] = resid_update(r[b + i], q[b + i], a);
+    for (int i = 0; i < N; ++i) v[i] = resid_update(v[i], t[i], a);
     if (cx > 0) v[0] = AddOp<VS>::add(resid_update(r[b - n3 + p], q[b - n3 + p], a), v[0]);
     if (cx + 1 < static_cast<uint32_t>(nx)) v[p] = AddOp<VS>::add(v[p], resid_update(r[b + n3], q[b + n3], a));
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (i < n) dst[b + i] = v[i];
+    line_st<N>(dst + b, v, LineVec<N, VS>::aligned(dst));
 }
 
 // r <- r - a q (a as above), the unfused form for vectors beyond 32-bit line indexing
@@ -565,6 +589,21 @@ template <class VS>
 static cudaError_t dss_typed(const Op &op, VS *v, int flags, cudaStream_t s, int first_axis = 0, int end_axis = 3,
                              int xtile = 0);
 
+// f(n as a compile-time constant) for n = 2..8
+template <class F>
+static void by_n(int n, F f)
+{
+    switch (n) {
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 5: return f(std::integral_constant<int, 5>{});
+    case 6: return f(std::integral_constant<int, 6>{});
+    case 7: return f(std::integral_constant<int, 7>{});
+    case 8: return f(std::integral_constant<int, 8>{});
+    }
+}
+
 // dst = S src (or S_bar src), src unchanged; src and dst must not overlap
 template <class VS>
 static cudaError_t dss_from_typed(const Op &op, const VS *src, VS *dst, int flags, cudaStream_t s)
@@ -576,12 +615,13 @@ static cudaError_t dss_from_typed(const Op &op, const VS *src, VS *dst, int flag
         return dss_typed(op, dst, flags, s, 0);
     }
     const uint32_t nlines = (uint32_t)(op.L / op.n);
-    if (flags == CW_DSS_AVERAGE)
-        dss_x_from_kernel<VS, true><<<(nlines + 255) / 256, 256, 0, s>>>(src, dst, m.nx, op.p, nlines,
-                                                                         FastDiv::make(op.n * op.n), FastDiv::make(m.nx));
-    else
-        dss_x_from_kernel<VS, false><<<(nlines + 255) / 256, 256, 0, s>>>(src, dst, m.nx, op.p, nlines,
-                                                                          FastDiv::make(op.n * op.n), FastDiv::make(m.nx));
+    auto run = [&](auto N) {
+        const FastDiv fx = FastDiv::make(m.nx);
+        if (flags == CW_DSS_AVERAGE)
+            dss_x_from_kernel<N(), VS, true><<<(nlines + 255) / 256, 256, 0, s>>>(src, dst, m.nx, nlines, fx);
+        else dss_x_from_kernel<N(), VS, false><<<(nlines + 255) / 256, 256, 0, s>>>(src, dst, m.nx, nlines, fx);
+    };
+    by_n(op.n, run);
     return dss_typed(op, dst, flags, s, 1);
 }
 
@@ -595,10 +635,29 @@ static cudaError_t dss_from_axpy_typed(const Op &op, VS *r, const VS *q, const d
         return dss_from_typed(op, static_cast<const VS *>(r), dst, CW_DSS_SUM, s);
     }
     const uint32_t nlines = (uint32_t)(op.L / op.n);
-    dss_x_axpy_kernel<VS><<<(nlines + 255) / 256, 256, 0, s>>>(r, q, alpha, active, dst, op.mesh->nx, op.p, nlines,
-                                                                 FastDiv::make(op.n * op.n), FastDiv::make(op.mesh->nx));
+    by_n(op.n, [&](auto N) {
+        dss_x_axpy_kernel<N(), VS><<<(nlines + 255) / 256, 256, 0, s>>>(r, q, alpha, active, dst, op.mesh->nx, nlines,
+                                                                        FastDiv::make(op.mesh->nx));
+    });
     if (x_only) return cudaGetLastError();
     return dss_typed(op, dst, CW_DSS_SUM, s, 1);
+}
+
+cudaError_t dss_average_from_scaled(const Op &op, const void *b, const void *d, void *dst, cudaStream_t s)
+{
+    const uint32_t nlines = (uint32_t)(op.L / op.n);
+    by_n(op.n, [&](auto N) {
+        const FastDiv fx = FastDiv::make(op.mesh->nx);
+        const unsigned g = (nlines + 255) / 256;
+        if (vec_elem_size(op.prec) == 8)
+            dss_x_scale_kernel<N(), double><<<g, 256, 0, s>>>(static_cast<const double *>(b), static_cast<const double *>(d),
+                                                              static_cast<double *>(dst), op.mesh->nx, nlines, fx);
+        else
+            dss_x_scale_kernel<N(), float><<<g, 256, 0, s>>>(static_cast<const float *>(b), static_cast<const float *>(d),
+                                                             static_cast<float *>(dst), op.mesh->nx, nlines, fx);
+    });
+    if (vec_elem_size(op.prec) == 8) return dss_typed(op, static_cast<double *>(dst), CW_DSS_AVERAGE, s, 1);
+    return dss_typed(op, static_cast<float *>(dst), CW_DSS_AVERAGE, s, 1);
 }
 
 cudaError_t dss_from_axpy(const Op &op, void *r, const void *q, const double *alpha, const int *active, void *dst,

@@ -22,6 +22,7 @@
 #include <type_traits>
 
 #include "cw_arith.cuh"
+#include "cw_line.cuh"
 #include "cw_tma.cuh"
 
 namespace cw {
@@ -554,14 +555,22 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         T v[N], w[N], u[N], acc[N], gx[N], gy[N], gz[N];
         // (1) x-line (j,k) = (ra, rb): N contiguous values of the cell, contracted with B along x
         {
+            VS xl[N];
+            bool have = act;
             if (x_smem) {  // a thread whose wait expired reads nothing staged
+                have = x_ok;
+                if (x_ok) LineVec<N, VS>::ld(xs + N * r, xl);
+            } else if (act) {
+                const VS *xg = x + cell * N3 + N * r;
+                if (LineVec<N, VS>::aligned(x)) {
+                    LineVec<N, VS>::ld_nc(xg, xl);
+                } else {
 #pragma unroll
-                for (int m = 0; m < N; ++m) v[m] = x_ok ? Ar::from(xs[N * r + m]) : Ar::zero();
-            } else {
-                const VS *xg = x + (act ? cell : 0) * N3 + N * r;
-#pragma unroll
-                for (int m = 0; m < N; ++m) v[m] = act ? Ar::from(ldg_nc(xg + m)) : Ar::zero();
+                    for (int m = 0; m < N; ++m) xl[m] = ldg_nc(xg + m);
+                }
             }
+#pragma unroll
+            for (int m = 0; m < N; ++m) v[m] = have ? Ar::from(xl[m]) : Ar::zero();
             sweep<N, Ar, 0, NRM>(tab, v, w);
             CW_TST(0, xi, 1, w);
         }
@@ -784,52 +793,38 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         {
             CW_TLD(0, xi, 1, v);
             sweep<N, Ar, 1, NRM>(tab, v, w);
-            if constexpr (SMOOTH) {
-                VS nv[N];
-                const int64_t o = (act ? cell : 0) * N3 + N * r;
+            VS nv[N];  // the values to store
+            const bool yvec = LineVec<N, VS>::aligned(y);
+            const int64_t o = (act ? cell : 0) * N3 + N * r;
 #pragma unroll
-                for (int m = 0; m < N; ++m) {
-                    VS av;
-                    Ar::to(av, w[m]);
-                    nv[m] = act ? y[o + m] + sd[o + m] * (sb[o + m] - av) : VS(0);
-                }
-                VS *exl = reinterpret_cast<VS *>(S0 + RS), *exr = exl + CPB * N2;  // buffer 1 is free
+            for (int m = 0; m < N; ++m) Ar::to(nv[m], w[m]);
+            if constexpr (SMOOTH) {
+                VS yl[N], bl[N], dl[N];
+                line_ld<N>(y + o, yl, yvec);
+                line_ld<N>(sb + o, bl, LineVec<N, VS>::aligned(sb));
+                line_ld<N>(sd + o, dl, LineVec<N, VS>::aligned(sd));
+#pragma unroll
+                for (int m = 0; m < N; ++m) nv[m] = act ? yl[m] + dl[m] * (bl[m] - nv[m]) : VS(0);
+            }
+            if (SMOOTH || asm_nx > 0) {  // kernel-uniform: the x-interfaces inside the tile
+                // buffer 1 is free: its last reads precede the first barrier of step (5)
+                VS *exl = reinterpret_cast<VS *>(S0 + RS), *exr = exl + CPB * N2;
                 exl[c * N2 + r] = nv[0];
                 exr[c * N2 + r] = nv[N - 1];
                 __syncthreads();
                 if (act) {
                     const int64_t ix = cell % asm_nx;
-                    if (c + 1 < cpt && cell + 1 < ncells && ix + 1 < asm_nx)
-                        nv[N - 1] = AddOp<VS>::add(nv[N - 1], exl[(c + 1) * N2 + r]) * VS(0.5);
-                    if (c > 0 && ix > 0) nv[0] = AddOp<VS>::add(exr[(c - 1) * N2 + r], nv[0]) * VS(0.5);
-#pragma unroll
-                    for (int m = 0; m < N; ++m) y[o + m] = nv[m];
+                    if (c + 1 < cpt && cell + 1 < ncells && ix + 1 < asm_nx) {
+                        nv[N - 1] = AddOp<VS>::add(nv[N - 1], exl[(c + 1) * N2 + r]);
+                        if constexpr (SMOOTH) nv[N - 1] = nv[N - 1] * VS(0.5);
+                    }
+                    if (c > 0 && ix > 0) {
+                        nv[0] = AddOp<VS>::add(exr[(c - 1) * N2 + r], nv[0]);
+                        if constexpr (SMOOTH) nv[0] = nv[0] * VS(0.5);
+                    }
                 }
-            } else if (asm_nx > 0) {  // kernel-uniform
-                VS o0, o1;
-                Ar::to(o0, w[0]);
-                Ar::to(o1, w[N - 1]);
-                // the S1 buffer is free: its last reads precede the first barrier of step (5)
-                VS *exl = reinterpret_cast<VS *>(S0 + RS), *exr = exl + CPB * N2;
-                exl[c * N2 + r] = o0;
-                exr[c * N2 + r] = o1;
-                __syncthreads();
-                if (act) {
-                    const int64_t ix = cell % asm_nx;
-                    if (c + 1 < cpt && cell + 1 < ncells && ix + 1 < asm_nx)
-                        o1 = AddOp<VS>::add(o1, exl[(c + 1) * N2 + r]);
-                    if (c > 0 && ix > 0) o0 = AddOp<VS>::add(exr[(c - 1) * N2 + r], o0);
-                    VS *yc = y + cell * N3 + N * r;
-                    yc[0] = o0;
-#pragma unroll
-                    for (int m = 1; m < N - 1; ++m) Ar::to(yc[m], w[m]);
-                    yc[N - 1] = o1;
-                }
-            } else if (act) {
-                VS *yc = y + cell * N3 + N * r;
-#pragma unroll
-                for (int m = 0; m < N; ++m) Ar::to(yc[m], w[m]);
             }
+            if (act) line_st<N>(y + o, nv, yvec);
         }
     }
 }
@@ -971,9 +966,18 @@ __global__ void __launch_bounds__(N *N *CPB) apply_affine_kernel(const VS *__res
     T v[N], P[N], Q[N];
     // x-line: P = M_x u, Q = K_x u
     {
-        const VS *xc = x + (act ? cell : 0) * N3 + N * r;
+        VS xl[N];
+        if (act) {
+            const VS *xc = x + cell * N3 + N * r;
+            if (LineVec<N, VS>::aligned(x)) {
+                LineVec<N, VS>::ld_nc(xc, xl);
+            } else {
 #pragma unroll
-        for (int m = 0; m < N; ++m) v[m] = act ? Ar::from(ldg_nc(xc + m)) : Ar::zero();
+                for (int m = 0; m < N; ++m) xl[m] = ldg_nc(xc + m);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < N; ++m) v[m] = act ? Ar::from(xl[m]) : Ar::zero();
         contract<N, false, Ar>(tab.M, v, P);
         CW_STX(s0, P);
         if (HAS_K) {

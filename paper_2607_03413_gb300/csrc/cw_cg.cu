@@ -32,6 +32,7 @@
 #include "cw_arith.cuh"
 #include "cw_index.cuh"
 #include "cw_internal.h"
+#include "cw_line.cuh"
 
 namespace cw {
 
@@ -449,35 +450,6 @@ __global__ void __launch_bounds__(kRedThreads) k_precond_fin(V *__restrict__ r, 
     last_block_finalize(part, scal, flags, stage);
 }
 
-// Line access of the fused kernel below: N consecutive values; one 16-byte access for N = 4 floats
-// (every line start there is 16-byte aligned: lines are 16 bytes apart and the partner offsets are
-// multiples of 4 floats).
-template <int N, class V>
-struct LineIO {
-    static __device__ __forceinline__ void ld(const V *p, V (&v)[N])
-    {
-#pragma unroll
-        for (int m = 0; m < N; ++m) v[m] = p[m];
-    }
-    static __device__ __forceinline__ void st(V *p, const V (&v)[N])
-    {
-#pragma unroll
-        for (int m = 0; m < N; ++m) p[m] = v[m];
-    }
-};
-template <>
-struct LineIO<4, float> {
-    static __device__ __forceinline__ void ld(const float *p, float (&v)[4])
-    {
-        const float4 t = *reinterpret_cast<const float4 *>(p);
-        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
-    }
-    static __device__ __forceinline__ void st(float *p, const float (&v)[4])
-    {
-        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    }
-};
-
 // The y and z passes of the DSS fused with the preconditioner: w holds S_x r' (x pass done, from
 // dss_from_axpy); every x-line gathers its y-partner, z-partner and yz-partner lines and sums them in
 // the passes' order ((own + y) + (z + zy), each copy the same tree, so all copies agree and the result
@@ -492,7 +464,7 @@ __global__ void __launch_bounds__(kRedThreads) k_precond_yz_fin(
 {
     if (stage == STAGE_RHO && flags[F_DONE]) return;  // an iteration after convergence
     constexpr int P = N - 1, N2 = N * N, N3 = N2 * N;
-    using IO = LineIO<N, V>;
+    using IO = LineVec<N, V>;  // solver vectors start at cudaMalloc allocations: every line is aligned
     const int sx = nx * N3, sxy = nx * ny * N3;  // < L < 2^31
     df64 a1{0.0f, 0.0f}, a2{0.0f, 0.0f};
     for (uint32_t l = blockIdx.x * blockDim.x + threadIdx.x; l < nlines; l += gridDim.x * blockDim.x) {
@@ -614,13 +586,15 @@ static cudaError_t apply_by_kind(const Op &op, int ak, const void *x, void *y, c
 }
 
 // whether q = A p can carry the <p, q> partials in its epilogue (curved cells, default tile and
-// TMA staging, double-float or FP32 arithmetic)
+// staging, double-float or FP32 arithmetic)
 static bool apply_dot_ok(const Op &op, int ak)
 {
     if (ak == AK_NATIVE) return false;
-    // curved stored metric: the TMA-staged default; recomputed metric: its default (input staged)
-    if (op.geom == CW_GEOM_METRIC ? op.stage != 1 : op.geom != CW_GEOM_RECOMPUTE) return false;
-    if (op.cpb != 0 && op.cpb != tile_cells(op.n, prec_f32_arith(op.prec))) return false;  // not the default tile
+    // curved stored metric: the staged variants; recomputed metric: its default (input staged)
+    const bool f32 = prec_f32_arith(op.prec);
+    if (op.geom == CW_GEOM_METRIC ? op.stage != 1 && op.stage != default_stage(op.n, f32) : op.geom != CW_GEOM_RECOMPUTE)
+        return false;
+    if (op.cpb != 0 && !default_cells(op.n, f32, true)) return false;  // not the default tile
     return op.prec == CW_PREC_F64 || op.prec == CW_PREC_F32 || op.prec == CW_PREC_F32_BF16G;
 }
 

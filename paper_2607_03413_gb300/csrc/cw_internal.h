@@ -31,11 +31,11 @@ __host__ __device__ constexpr int tile_cells(int n, bool f32)
 }
 
 // Staging mode a stored-metric operator starts with (op.stage). FP32 arithmetic: 1 (input and metric
-// tiles by TMA). Double-float: 1 or, where the metric tile's shared memory costs too many CTAs per SM,
-// 2 (each thread's metric entries two points ahead by 8-byte cp.async): Laplace at 51^3 Q5 866 us against
-// 985, 35^3 Q7 710 against 721, 64^3 Q4 K+M 817 against 823; at 78^3 Q3 565 against 533 and 42^3 Q6 857
-// against 784 mode 1 stays.
-__host__ __device__ constexpr int default_stage(int n, bool f32) { return !f32 && (n == 5 || n == 6 || n == 8) ? 2 : 1; }
+// tiles by TMA). Double-float: 1, but 2 (each thread's metric entries two points ahead by 8-byte
+// cp.async) at n = 6, where the staged metric leaves 3 CTAs of 4.5 warps per SM. Laplace, mode 1 / 2 us:
+// 51^3 Q5 985 / 866, but 99^3 Q2 472 / 531, 78^3 Q3 526 / 547, 64^3 Q4 779 / 795, 42^3 Q6 787 / 846,
+// 35^3 Q7 694 / 735.
+__host__ __device__ constexpr int default_stage(int n, bool f32) { return !f32 && n == 6 ? 2 : 1; }
 // Whether an operator starts with the alternative tile (half the default): FP32 vectors at n = 7, where
 // 8 cells are 2 CTAs per SM (42^3 Q6 Laplace 175 us with 4 cells, 281 with 8; BF16 182 with 8, 216 with 4).
 __host__ __device__ constexpr bool default_cells(int n, bool f32, bool vec4) { return f32 && n == 7 && vec4; }
@@ -178,6 +178,8 @@ cudaError_t mg_smooth_launch_f32(const Op &op, void *u, const void *b, const voi
 // the averaging DSS (every pass halves its pair sums, so no separate division by the valence) with the
 // x pass restricted to the interfaces between tiles of xtile cells (0: all)
 cudaError_t dss_average_launch(const Op &op, void *v, cudaStream_t s, int xtile);
+// dst = S_bar (d b) per copy (FP32 or FP64 vectors, op.L < 2^31): the product and the x averages in one pass
+cudaError_t dss_average_from_scaled(const Op &op, const void *b, const void *d, void *dst, cudaStream_t s);
 struct MgHier;
 // u = MG(b): one V-cycle on the finest level from a zero initial guess (enqueue only)
 cudaError_t mg_vcycle_zero(MgHier &h, const void *b, void *u, cudaStream_t s);

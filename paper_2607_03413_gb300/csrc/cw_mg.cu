@@ -169,7 +169,7 @@ static bool fused_sweep(const MgHier &h, const Op &op)
 }
 
 // `sweeps` sweeps of Algorithm smoother_fused: u <- S_bar (u + D_hat (b - A u)). The first sweep from
-// u = 0 (zero) is u = S_bar D_hat b. A fused sweep is one operator launch whose epilogue applies the
+// u = 0 (zero) is u = S_bar D_hat b, the product formed in the first averaging pass. A fused sweep is one operator launch whose epilogue applies the
 // update and the x averages inside its tiles, then the x pass between tiles and the y and z passes of
 // the averaging DSS; otherwise operator, update kernel and the three averaging passes.
 template <class VS>
@@ -183,7 +183,10 @@ static cudaError_t smooth_t(const MgHier &h, int l, const VS *b, VS *u, int swee
     for (int k = 0; k < sweeps; ++k) {
         cudaError_t e;
         int xtile = 0;
-        if (zero && k == 0) {
+        if (zero && k == 0 && op.L < ((int64_t)1 << 31)) {
+            if ((e = dss_average_from_scaled(op, b, dh, u, s)) != cudaSuccess) return e;
+            continue;
+        } else if (zero && k == 0) {
             k_jacobi_zero<VS><<<vgrid(op.L), 256, 0, s>>>(u, b, dh, op.L);
         } else if (fused) {
             e = h.prec == CW_PREC_F64 ? mg_smooth_launch_df(op, u, b, dh, s, &xtile)

@@ -21,12 +21,11 @@ struct TabTransfer {
     C P[2][N][N];  // P[b][i][a] = l_a((g_i + b) / 2)
 };
 
-// coarse cells per CTA of the transfer kernels (threads: 8 N^2 CP for prolongation, 4 N^2 CP for
-// restriction)
+// coarse cells per CTA of the transfer kernels (4 N^2 CP threads)
 template <int N>
 constexpr int prolong_cp()
 {
-    return N == 2 ? 8 : N == 3 ? 4 : N == 4 ? 2 : 1;
+    return N == 2 ? 16 : N == 3 ? 8 : N == 4 ? 4 : N <= 6 ? 2 : 1;
 }
 template <int N>
 constexpr int restrict_cp()
@@ -44,10 +43,14 @@ __device__ __forceinline__ int64_t child_cell(int64_t e, int nx, int ny, int ch)
 // uf|K_c (+)= (P_bz x P_by x P_bx) uc|K for every child c of the coarse cells of this CTA.
 // ADD: add into uf (the V-cycle's u += P e), else overwrite (Algorithm prolongation into a zeroed
 // vector). nx, ny: coarse cells per direction. The axes are contracted z, y, x, so that the last phase
-// owns whole x-lines of a child: each thread writes N contiguous values, consecutive threads the
-// consecutive lines of one child (the Kronecker factors commute).
+// owns whole x-lines of the children (the Kronecker factors commute). A thread contracts each line it
+// reads with both child matrices, which makes every coefficient an immediate constant operand and halves
+// the shared-memory reads: N^2, 2 N^2 and 4 N^2 lines per parent in the three phases, two results each;
+// the last phase moves whole lines of the fine vector (LineVec). With one thread per fine line that picked
+// its matrices by lane (indexed constant loads) and moved single values, 64^3 Q3 FP32 took 92 us (read and
+// write u: 21 us at the measured copy rate).
 template <int N, int CP, class Ar, class VS, bool ADD>
-__global__ void __launch_bounds__(8 * N * N * CP) prolong_kernel(const VS *__restrict__ uc, VS *__restrict__ uf,
+__global__ void __launch_bounds__(4 * N * N * CP) prolong_kernel(const VS *__restrict__ uc, VS *__restrict__ uf,
                                                                   int nx, int ny, int64_t ncoarse,
                                                                   TabTransfer<N, typename Ar::C> tab)
 {
@@ -60,15 +63,19 @@ __global__ void __launch_bounds__(8 * N * N * CP) prolong_kernel(const VS *__res
     const int t = threadIdx.x;
     const int64_t e0 = static_cast<int64_t>(blockIdx.x) * CP;
     const int64_t nval = ncoarse * N3;
-    // this thread's fine x-line (last phase): with ADD its old values are loaded first, so that the
-    // read overlaps the three contraction phases instead of stalling the store
-    const int xc = t / (8 * N2), xr = t - xc * 8 * N2, xch = xr / N2, xjk = xr - xch * N2;
+    const bool vec = LineVec<N, VS>::aligned(uf);
+    // this thread's two fine x-lines (last phase: line (j, k) of the children bx = 0, 1 of quarter
+    // by + 2 bz, adjacent fine cells); with ADD their old values are loaded first, so that the read
+    // overlaps the contraction phases instead of stalling the store
+    const int xc = t / (4 * N2), xr = t - xc * 4 * N2, xq = xr / N2, xjk = xr - xq * N2;
     const int64_t xe = e0 + xc;
-    VS *dst = xe < ncoarse ? uf + child_cell(xe, nx, ny, xch) * N3 + xjk * N : nullptr;
-    VS old[N];
+    VS *dst = xe < ncoarse ? uf + child_cell(xe, nx, ny, 2 * xq) * N3 + xjk * N : nullptr;
+    VS old[2][N];
     if constexpr (ADD) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) old[i] = dst ? dst[i] : VS(0);
+        if (dst) {
+            line_ld<N>(dst, old[0], vec);
+            line_ld<N>(dst + N3, old[1], vec);
+        }
     }
     for (int k = t; k < CP * N3; k += blockDim.x) {
         const int64_t g = e0 * N3 + k;
@@ -76,36 +83,45 @@ __global__ void __launch_bounds__(8 * N * N * CP) prolong_kernel(const VS *__res
     }
     __syncthreads();
     T in[N], out[N];
-    if (t < CP * 2 * N2) {  // z: pencil (i, j) of parent c, child half bz
-        const int c = t / (2 * N2), r = t - c * 2 * N2, bz = r / N2, ij = r - bz * N2;
+    if (t < CP * N2) {  // z: pencil (i, j) of parent c, both child halves bz
+        const int c = t / N2, ij = t - c * N2;
 #pragma unroll
         for (int m = 0; m < N; ++m) in[m] = S0[c * N3 + ij + N2 * m];
-        contract<N, false, Ar>(tab.P[bz], in, out);
 #pragma unroll
-        for (int k = 0; k < N; ++k) S1[(c * 2 + bz) * N3 + ij + N2 * k] = out[k];
+        for (int bz = 0; bz < 2; ++bz) {
+            contract<N, false, Ar>(tab.P[bz], in, out);
+#pragma unroll
+            for (int k = 0; k < N; ++k) S1[(c * 2 + bz) * N3 + ij + N2 * k] = out[k];
+        }
     }
     __syncthreads();
-    if (t < CP * 4 * N2) {  // y: line (i, k) of the quarter q = by + 2 bz
-        const int c = t / (4 * N2), r = t - c * 4 * N2, q = r / N2, ik = r - q * N2;
-        const int i = ik % N, k = ik / N, by = q & 1, bz = q >> 1;
+    if (t < CP * 2 * N2) {  // y: line (i, k) of the half bz, both by
+        const int c = t / (2 * N2), r = t - c * 2 * N2, bz = r / N2, ik = r - bz * N2;
+        const int i = ik % N, k = ik / N;
 #pragma unroll
         for (int m = 0; m < N; ++m) in[m] = S1[(c * 2 + bz) * N3 + i + N * m + N2 * k];
-        contract<N, false, Ar>(tab.P[by], in, out);
 #pragma unroll
-        for (int j = 0; j < N; ++j) S2[(c * 4 + q) * N3 + i + N * j + N2 * k] = out[j];
+        for (int by = 0; by < 2; ++by) {
+            contract<N, false, Ar>(tab.P[by], in, out);
+#pragma unroll
+            for (int j = 0; j < N; ++j) S2[(c * 4 + by + 2 * bz) * N3 + i + N * j + N2 * k] = out[j];
+        }
     }
     __syncthreads();
-    {  // x: line (j, k) of child ch = bx + 2 by + 4 bz
+    {  // x: line (j, k) of the quarter, both bx
 #pragma unroll
-        for (int m = 0; m < N; ++m) in[m] = S2[(xc * 4 + (xch >> 1)) * N3 + xjk * N + m];
-        contract<N, false, Ar>(tab.P[xch & 1], in, out);
-        if (dst) {
+        for (int m = 0; m < N; ++m) in[m] = S2[(xc * 4 + xq) * N3 + xjk * N + m];
 #pragma unroll
-            for (int i = 0; i < N; ++i) {
-                VS o;
-                Ar::to(o, out[i]);
-                if constexpr (ADD) dst[i] = old[i] + o;
-                else dst[i] = o;
+        for (int bx = 0; bx < 2; ++bx) {
+            contract<N, false, Ar>(tab.P[bx], in, out);
+            if (dst) {
+                VS o[N];
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    Ar::to(o[i], out[i]);
+                    if constexpr (ADD) o[i] = old[bx][i] + o[i];
+                }
+                line_st<N>(dst + bx * N3, o, vec);
             }
         }
     }
@@ -189,9 +205,10 @@ __global__ void __launch_bounds__(4 * N * N * CP) restrict_kernel(const VS *__re
             for (int a = 0; a < N; ++a) acc[a] = bx ? Ar::add(acc[a], out[a]) : out[a];
         }
         if (e < ncoarse) {
-            VS *dst = bc + e * N3 + jk * N;
+            VS o[N];
 #pragma unroll
-            for (int a = 0; a < N; ++a) Ar::to(dst[a], acc[a]);
+            for (int a = 0; a < N; ++a) Ar::to(o[a], acc[a]);
+            line_st<N>(bc + e * N3 + jk * N, o, LineVec<N, VS>::aligned(bc));
         }
     }
 }
@@ -224,10 +241,10 @@ cudaError_t prolong_n(const Op &coarse, const void *uc, void *uf, bool add, cuda
     const VS *in = static_cast<const VS *>(uc);
     VS *out = static_cast<VS *>(uf);
     if (add)
-        prolong_kernel<N, CP, Ar, VS, true><<<grid, 8 * N * N * CP, smem, s>>>(in, out, coarse.mesh->nx, coarse.mesh->ny,
+        prolong_kernel<N, CP, Ar, VS, true><<<grid, 4 * N * N * CP, smem, s>>>(in, out, coarse.mesh->nx, coarse.mesh->ny,
                                                                               coarse.E, tab);
     else
-        prolong_kernel<N, CP, Ar, VS, false><<<grid, 8 * N * N * CP, smem, s>>>(in, out, coarse.mesh->nx,
+        prolong_kernel<N, CP, Ar, VS, false><<<grid, 4 * N * N * CP, smem, s>>>(in, out, coarse.mesh->nx,
                                                                                coarse.mesh->ny, coarse.E, tab);
     return cudaGetLastError();
 }
