@@ -488,6 +488,56 @@ static cudaError_t dss_node_typed(const Op *const *ops, const int64_t *off, cons
     return cudaGetLastError();
 }
 
+// The y and z passes of Algorithm struct_dss in one launch, x-line by x-line: the lowest copy of a line on an
+// interior y- or z-face (2 copies, 4 on the edges between them) owns it; its thread reads the copies, sums them
+// in the passes' order (y pairs, then z; HALF: each sum halved) and writes them back, bit-identical to the
+// passes and in place. One thread per line (j, p) or (p, k) of a cell. Bound by the 32-byte sectors the face
+// lines touch, which the two passes fetch and write twice between them.
+template <int N, class VS, bool HALF>
+__global__ void __launch_bounds__(256) dss_yz_kernel(VS *__restrict__ v, int nx, int ny, int nz, uint32_t nthr,
+                                                     FastDiv fd_m, FastDiv fd_nx, FastDiv fd_ny, bool vec)
+{
+    const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+    if (t >= nthr) return;
+    constexpr int P = N - 1, N2 = N * N;
+    constexpr int64_t N3 = N * N * N;
+    const uint32_t e = fd_m.div(t);
+    const int m = static_cast<int>(t - e * (2 * N - 1));  // lines (m, P) for m < N, then (P, m - N)
+    const int j = m < N ? m : P, k = m < N ? P : m - N;
+    const uint32_t row = fd_nx.div(e), cz = fd_ny.div(row);
+    const int cy = static_cast<int>(row - cz * static_cast<uint32_t>(ny));
+    const bool hy = j == P && cy + 1 < ny, hz = k == P && static_cast<int>(cz) + 1 < nz;
+    if (!(hy || hz) || (j == 0 && cy > 0) || (k == 0 && cz > 0)) return;
+    const int64_t dy = N3 * nx - P * N, dz = N3 * nx * ny - P * N2;
+    VS *o = v + e * N3 + N * (j + N * k);
+    auto add = [](VS (&a)[N], const VS (&b)[N]) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            a[i] = AddOp<VS>::add(a[i], b[i]);
+            if constexpr (HALF) a[i] = half_of(a[i]);
+        }
+    };
+    VS s[N], b[N];
+    line_ld<N>(o, s, vec);
+    if (hy) {
+        line_ld<N>(o + dy, b, vec);
+        add(s, b);
+    }
+    if (hz) {
+        VS c[N];
+        line_ld<N>(o + dz, c, vec);
+        if (hy) {
+            line_ld<N>(o + dz + dy, b, vec);
+            add(c, b);
+        }
+        add(s, c);
+        line_st<N>(o + dz, s, vec);
+        if (hy) line_st<N>(o + dz + dy, s, vec);
+    }
+    line_st<N>(o, s, vec);
+    if (hy) line_st<N>(o + dy, s, vec);
+}
+
 // dst = src with the x pass of Algorithm struct_dss applied: an entry on an interior x-face adds its
 // partner copy in the neighbouring cell, every other entry is copied (out of place, so the read of
 // a partner never sees an updated value). Replaces a copy and an in-place x pass with one pass.
@@ -689,6 +739,19 @@ cudaError_t dss_from_f64(const Op &op, const double *src, double *dst, int flags
     return dss_from_typed(op, src, dst, flags, s);
 }
 
+// Where one launch does the y and z passes, by measurement (us per DSS including its x pass, one launch /
+// passes): lines of even n are moved in wide accesses, odd ones value by value. FP32 Q3 106/111 at 32e6
+// entries, 31/29 at 8e6, Q5 88/94, Q7 75/87, but Q4 118/103; BF16 Q3 58/88, Q5 55/68, Q7 44/56, Q4 111/76. In FP64 the
+// passes are bound by their FP64 additions and the one launch pays in large sums only: Q3 164/182, Q5
+// 147/162 at 32e6 entries, 43/42, 34/32 at 8e6, Q7 133/129; averages 239/184.
+template <class VS>
+static bool dss_yz_one_launch(const Op &op, int flags)
+{
+    if (op.n % 2 || (op.mesh->ny < 2 && op.mesh->nz < 2) || op.E * (2 * op.n - 1) >= ((int64_t)1 << 31)) return false;
+    if (sizeof(VS) < 8) return true;
+    return flags == CW_DSS_SUM && (op.n == 4 || op.n == 6) && op.L >= ((int64_t)1 << 24);
+}
+
 template <class VS>
 static cudaError_t dss_typed(const Op &op, VS *v, int flags, cudaStream_t s, int first_axis, int end_axis, int xtile)
 {
@@ -701,6 +764,18 @@ static cudaError_t dss_typed(const Op &op, VS *v, int flags, cudaStream_t s, int
         return dss_node_typed(&o, nullptr, &xt, 1, v, flags, s);
     }
     for (int ax = first_axis; ax < end_axis; ++ax) {
+        if (ax == 1 && end_axis == 3 && dss_yz_one_launch<VS>(op, flags)) {
+            const uint32_t nthr = (uint32_t)(op.E * (2 * op.n - 1));
+            by_n(op.n, [&](auto N) {
+                const FastDiv fm = FastDiv::make(2 * N() - 1), fx = FastDiv::make(m.nx), fy = FastDiv::make(m.ny);
+                const bool vec = LineVec<N(), VS>::aligned(v);
+                if (flags == CW_DSS_AVERAGE)
+                    dss_yz_kernel<N(), VS, true><<<(nthr + 255) / 256, 256, 0, s>>>(v, m.nx, m.ny, m.nz, nthr, fm, fx, fy, vec);
+                else
+                    dss_yz_kernel<N(), VS, false><<<(nthr + 255) / 256, 256, 0, s>>>(v, m.nx, m.ny, m.nz, nthr, fm, fx, fy, vec);
+            });
+            break;
+        }
         if (dims[ax] < 2) continue;
         // in-face coordinates: a = lower of the two other axes (x-index part), b = the other (grid y)
         const int a = (ax == 0) ? 1 : 0, b = (ax == 2) ? 1 : 2;

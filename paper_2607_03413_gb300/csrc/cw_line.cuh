@@ -21,7 +21,7 @@ struct LineVec {
                                  std::conditional_t<VB == 8, uint2, std::conditional_t<VB == 4, uint32_t, uint16_t>>>;
     static_assert(VB >= (int)sizeof(V), "a line is a whole number of accesses");
 
-    static __device__ __forceinline__ bool aligned(const void *base)
+    static __host__ __device__ __forceinline__ bool aligned(const void *base)
     {
         return (reinterpret_cast<uintptr_t>(base) & (VB - 1)) == 0;
     }
