@@ -143,16 +143,37 @@ def _check(st, where):
         raise CwError(st, where)
 
 
+_torch = None  # imported at the first call that needs it
+_raw_stream = None
+
+
+def _get_torch():
+    global _torch, _raw_stream
+    if _torch is None:
+        import torch
+        # the current stream's handle without building a Stream object (3 us of a 9 us call)
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+            (lambda device: torch.cuda.current_stream(device).cuda_stream)
+        _torch = torch
+    return _torch
+
+
 def _stream(stream=None):
     if stream is not None:
         return ctypes.c_void_p(stream)
-    import torch
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    device = (_torch or _get_torch()).cuda.current_device()
+    return ctypes.c_void_p(_raw_stream(device))
 
 
 def _ptr(t):
     if t is None:
         return None
+    if _torch is not None and type(t) is _torch.Tensor:  # the common case, without attribute probes
+        if not t.is_cuda:
+            raise ValueError("expected a CUDA tensor")
+        if not t.is_contiguous():
+            raise ValueError("expected a contiguous tensor")
+        return ctypes.c_void_p(t.data_ptr())
     if hasattr(t, "data_ptr"):
         if hasattr(t, "is_cuda") and not t.is_cuda:
             raise ValueError("expected a CUDA tensor")
@@ -490,8 +511,7 @@ class Operator:
 
     @property
     def vec_dtype(self):
-        import torch
-        return getattr(torch, _VEC_DTYPE[self.prec])
+        return getattr(_torch or _get_torch(), _VEC_DTYPE[self.prec])
 
     def empty(self):
         import torch
