@@ -252,21 +252,44 @@ struct Lines {
 // cells (2.4x the L2 store sectors) and was slower. Double-float and FP64 tiles (8-byte elements)
 // keep odd row pitches with lines in thread order: their kernel is bound by the FP32 pipes, and 22 %
 // fewer wavefronts changed nothing in its time.
+//
+// n = 4 and 8 in 4-byte elements: dense buffers with a swizzle instead of pitches. Element (i, j, k) of cell
+// slot c sits at word D(c) ^ A(i) ^ B(j) ^ C(k) (tile_swz): the 16-byte chunks of an x-line keep their four
+// elements together, and the chunk bits below 32 words are mixed so that in every warp the 32 x-lines (as
+// 16-byte accesses, 8 lanes at a time), the 32 y-lines and the 32 z-pencils each cover all banks: no access of
+// the apply has a conflict. With the pitches above (and dealt lines) an n = 4 apply took 1.54 shared-memory
+// wavefronts per value (0.94 without conflicts) and kept the L1 data path 91 % busy.
+__host__ __device__ constexpr bool tile_swizzled(int N, int ESZ, bool allow_remap)
+{
+    return allow_remap && ESZ == 4 && (N == 4 || N == 8);
+}
+template <int N>
+struct TileSwz {  // N = 4: a warp holds two cells (c odd and even); N = 8: half a cell
+    static __host__ __device__ constexpr int A(int i) { return i; }
+    static __host__ __device__ constexpr int B(int j)
+    {
+        return N == 4 ? 4 * j : (4 * (j >> 2)) ^ (8 * (j & 3)) ^ (32 * (j >> 2));
+    }
+    static __host__ __device__ constexpr int C(int k)
+    {
+        return N == 4 ? (4 * (k >> 1)) ^ (16 * (k & 1)) ^ (32 * (k >> 1)) : (8 * (k & 3)) ^ (64 * k);
+    }
+    static __host__ __device__ constexpr int D(int c) { return N == 4 ? 64 * c ^ ((c & 1) ? 24 : 0) : 512 * c; }
+};
 struct TileGeom {
     int pi, pp, cs;  // row pitch, plane pitch, cell stride (elements)
     bool deal_x, deal_y;
 };
 __host__ __device__ constexpr TileGeom tile_geom(int N, int CPB, int ESZ, bool allow_remap)
 {
+    if (tile_swizzled(N, ESZ, allow_remap)) return {N, N * N, N * N * N, false, false};
     if (allow_remap && ESZ == 4) {
         switch (N * 1000 + CPB) {
         case 2016: case 2032: case 2064: return {2, 6, 12, false, true};
         case 3008: case 3016: case 3032: return {3, 10, 41, true, true};
-        case 4004: case 4008: return {4, 19, 80, true, true};
         case 5004: case 5008: return {5, 33, 185, true, true};
         case 6002: case 6004: case 6008: return {6, 37, 228, true, true};
         case 7004: case 7008: return {7, 73, 529, true, true};
-        case 8002: return {8, 66, 528, true, true};
         default: break;
         }
     }
@@ -331,16 +354,49 @@ constexpr bool line_map_is_bijection()
 template <int N, int CPB, int ESZ, bool REMAP>
 __device__ constexpr LineMap<N, CPB, ESZ> kLineMap = make_line_map<N, CPB, ESZ, REMAP>();
 
-// element m of a line in buffer R: x-line at offset o (stride 1), y-line (stride PI), z-pencil (PP)
-#define CW_TLD(R, o, st, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) v[m_] = S0[(R) * TL::RS + (o) + (st) * m_]
-#define CW_TST(R, o, st, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) S0[(R) * TL::RS + (o) + (st) * m_] = v[m_]
-
 #define CW_LDX(s, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) v[m_] = (s)[L::x(ra, rb, m_)]
 #define CW_LDY(s, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) v[m_] = (s)[L::y(ra, rb, m_)]
 #define CW_LDZ(s, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) v[m_] = (s)[L::z(ra, rb, m_)]
 #define CW_STX(s, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) (s)[L::x(ra, rb, m_)] = v[m_]
 #define CW_STY(s, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) (s)[L::y(ra, rb, m_)] = v[m_]
 #define CW_STZ(s, v) _Pragma("unroll") for (int m_ = 0; m_ < N; ++m_) (s)[L::z(ra, rb, m_)] = v[m_]
+
+// A thread's share of <x, A x>, accumulated in double-float. FP32 arithmetic: the products of two FP32 values
+// have no low parts to carry (10 operations each instead of 12), and those of the x- and y-derivatives run as
+// the two lanes of paired instructions with a sum of their own: 20 instructions per point instead of 36,
+// beside about 100 for the operator.
+struct DotAcc {
+    df64 s{0.0f, 0.0f};
+    float2 hi2 = make_float2(0.0f, 0.0f), lo2 = make_float2(0.0f, 0.0f);
+};
+__device__ __forceinline__ void dot_add(DotAcc &d, df64 a, df64 b) { df_mad(d.s, a, b); }
+__device__ __forceinline__ void dot_add(DotAcc &d, float a, float b)
+{
+    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+    float s, t;
+    two_sum(d.s.hi, p, s, t);
+    d.s.hi = s;
+    d.s.lo = __fadd_rn(d.s.lo, __fadd_rn(t, e));
+}
+__device__ __forceinline__ void dot_add2(DotAcc &d, df64 a, df64 b, df64 a2, df64 b2)
+{
+    df_mad(d.s, a, b);
+    df_mad(d.s, a2, b2);
+}
+__device__ __forceinline__ void dot_add2(DotAcc &d, float a, float b, float a2, float b2)
+{
+    const float2 x = make_float2(a, a2), y = make_float2(b, b2), p = __fmul2_rn(x, y);
+    const float2 e = __ffma2_rn(x, y, neg2(p));
+    float2 s, t;
+    two_sum2(d.hi2, p, s, t);
+    d.hi2 = s;
+    d.lo2 = __fadd2_rn(d.lo2, __fadd2_rn(t, e));
+}
+__device__ __forceinline__ double dot_value(const DotAcc &d)
+{
+    df64 t = df_add(d.s, df64{d.hi2.x, d.lo2.x});
+    return df_to_double(df_add(t, df64{d.hi2.y, d.lo2.y}));
+}
 
 // number of stored metric components per quadrature point for an operator kind
 __host__ __device__ constexpr int metric_ncomp(int kind) { return kind == 1 ? 6 : (kind == 2 ? 1 : 7); }
@@ -357,7 +413,8 @@ __host__ __device__ constexpr int metric_ncomp(int kind) { return kind == 1 ? 6 
 // STAGE 0: direct loads; 1: x and metric tiles staged in shared memory by TMA; 2: x tile staged by
 // TMA, metric tile prefetched into L2 by a bulk prefetch (a third of the shared memory of mode 1,
 // so more CTAs per SM), then read with direct loads; 3: the metric tile in shared memory or on its way
-// there (staged by the caller for several right-hand sides, gsm; gbar != nullptr: the copy completes
+// there (staged by the caller for several right-hand sides: gsm, gcs elements per cell; gbar != nullptr: the
+// copy completes
 // phase gphase of *gbar, waited for before the physics step), x read directly.
 // Line buffers of metric_tile: three for 4-byte elements; two for 8-byte ones (double-float and FP64
 // arithmetic), whose y-derivatives go back into buffer 0 after one more barrier: with the metric staged
@@ -378,11 +435,31 @@ constexpr bool metric_ring()
     return std::is_same<Ar, ArDF>::value && STAGE == 2 && !RC;
 }
 
+// Elements between the staged metrics of two cells beyond their own: at n = 4 in FP32 arithmetic the two cells
+// of a warp read the same banks (a cell's metric is a multiple of 32 words), so each cell gets 64 bytes more
+// and a bulk copy of its own.
+template <int N, class T, class GS>
+__host__ __device__ constexpr int metric_pad()
+{
+    return N == 4 && sizeof(T) == 4 ? 64 / (int)sizeof(GS) : 0;
+}
+// the bulk copies of a tile's metric (CPB cells of gc elements) into shared memory, by one thread
+template <int CPB, int PAD, class GS>
+__device__ __forceinline__ void metric_copy(GS *dst, const GS *src, int gc, uint64_t *bar)
+{
+    if constexpr (PAD == 0) {
+        bulk_g2s(dst, src, CPB * gc * sizeof(GS), bar);
+    } else {
+#pragma unroll
+        for (int c = 0; c < CPB; ++c) bulk_g2s(dst + c * (gc + PAD), src + c * gc, gc * sizeof(GS), bar);
+    }
+}
+
 template <int N, int CPB, class T, class GS, bool REMAP = true>
 __host__ __device__ constexpr size_t metric_smem_bytes(int nc, int stage)
 {
     constexpr size_t lb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), REMAP>::RS * sizeof(T);  // a multiple of 16
-    return stage == 1 ? lb + (CPB * nc * N * N * N * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 + (std::is_same<T, df64>::value ? kRing * nc * N * N * CPB * sizeof(GS) : 0) : lb;
+    return stage == 1 ? lb + (CPB * (nc * N * N * N + metric_pad<N, T, GS>()) * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 + (std::is_same<T, df64>::value ? kRing * nc * N * N * CPB * sizeof(GS) : 0) : lb;
 }
 
 // One tile of `cpt` consecutive cells starting at cell tile*cpt, worked by CPB cell slots of N*N
@@ -396,8 +473,8 @@ __host__ __device__ constexpr size_t metric_smem_bytes(int nc, int stage)
 // exchanged through shared memory and summed as that pass sums them); the interfaces between tiles
 // are left to the DSS.
 // RC: geo holds the trilinear coefficients (kTriCoef per cell) and the metric of every quadrature
-// point is recomputed from them (Sec. 6: J, det J, J^-1 at the point): G = (w / det J) [c_a . c_b]
-// with c_0 = J_eta x J_zeta, c_1 = J_zeta x J_xi, c_2 = J_xi x J_eta (the rows of det J J^-1), and
+// point is recomputed from them (Sec. 6: J, det J, J^-1 at the point), G = (w / det J) [c_a . c_b], applied
+// without forming it: G g = (w / det J) c_a . (sum_b c_b g_b), with c_0 = J_eta x J_zeta, c_1 = J_zeta x J_xi, c_2 = J_xi x J_eta (the rows of det J J^-1), and
 // the mass coefficient w det J.
 // SMOOTH (Algorithm smoother_fused in one pass over the operator's output): y aliases x (= u, updated
 // in place), and the stored value is u + D_hat (b - A u) (sb = b, sd = D_hat, cell-wise in the vector
@@ -426,10 +503,11 @@ template <int N, int CPB, class Ar, class VS, class GS, int STAGE, bool DOT = fa
           bool SMOOTH = false, bool REMAP = true>
 __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__restrict__ geo,
                                             int64_t ncells, int kind, const TabMetric<N, typename Ar::C> &tab,
-                                            int64_t tile, int cpt, unsigned char *smem_raw, df64 *dot = nullptr,
+                                            int64_t tile, int cpt, unsigned char *smem_raw, DotAcc *dot = nullptr,
                                             int asm_nx = 0, const VS *sb = nullptr, const VS *sd = nullptr,
                                             unsigned *status = nullptr, uint32_t dbg_extra = 0,
-                                            const GS *gsm = nullptr, uint64_t *gbar = nullptr, uint32_t gphase = 0)
+                                            const GS *gsm = nullptr, int gcs = 0, uint64_t *gbar = nullptr,
+                                            uint32_t gphase = 0)
 {
     static_assert(!(RC && STAGE == 1), "recomputed geometry has no metric tile to stage");
     // Double-float renormalisation of the intermediate values: kept where the operator serves the
@@ -464,6 +542,56 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         yo = yc * CS + (yr % N) + PP * (yr / N);
     }
 
+    // load / store of a line of buffer R (0, 1, 2): x-line (own: the thread's own cell), y-line, z-pencil
+    constexpr bool SW = tile_swizzled(N, sizeof(T), REMAP);
+    using Z = TileSwz<N>;
+    [[maybe_unused]] const int sx = Z::D(c) ^ Z::B(ra) ^ Z::C(rb), sy = Z::D(c) ^ Z::A(ra) ^ Z::C(rb);
+    [[maybe_unused]] const int sz = Z::D(c) ^ Z::A(ra) ^ Z::B(rb);
+    auto ldx = [&](int R, bool own, T(&v)[N]) {
+        const T *b = S0 + R * RS;
+        if constexpr (SW) {
+            T h[4];
+#pragma unroll
+            for (int m = 0; m < N; m += 4) {
+                LineVec<4, T>::ld(b + (sx ^ m), h);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[m + i] = h[i];
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < N; ++m) v[m] = b[(own ? xi : xo) + m];
+        }
+    };
+    auto stx = [&](int R, bool own, const T(&v)[N]) {
+        T *b = S0 + R * RS;
+        if constexpr (SW) {
+#pragma unroll
+            for (int m = 0; m < N; m += 4) {
+                const T h[4] = {v[m], v[m + 1], v[m + 2], v[m + 3]};
+                LineVec<4, T>::st(b + (sx ^ m), h);
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < N; ++m) b[(own ? xi : xo) + m] = v[m];
+        }
+    };
+    auto ldy = [&](int R, T(&v)[N]) {
+#pragma unroll
+        for (int m = 0; m < N; ++m) v[m] = S0[R * RS + (SW ? sy ^ Z::B(m) : yo + PI * m)];
+    };
+    auto sty = [&](int R, const T(&v)[N]) {
+#pragma unroll
+        for (int m = 0; m < N; ++m) S0[R * RS + (SW ? sy ^ Z::B(m) : yo + PI * m)] = v[m];
+    };
+    auto ldz = [&](int R, T(&v)[N]) {
+#pragma unroll
+        for (int m = 0; m < N; ++m) v[m] = S0[R * RS + (SW ? sz ^ Z::C(m) : zo + PP * m)];
+    };
+    auto stz = [&](int R, const T(&v)[N]) {
+#pragma unroll
+        for (int m = 0; m < N; ++m) S0[R * RS + (SW ? sz ^ Z::C(m) : zo + PP * m)] = v[m];
+    };
+
     // ---- tile staging (single right-hand side)
     bool x_smem = false, g_smem = false, x_ok = true;
     const VS *xs = nullptr;
@@ -473,7 +601,8 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
     if constexpr (STAGE == 1) {
         const size_t offg = NB * RS * sizeof(T);
         GS *sG = reinterpret_cast<GS *>(smem_raw + offg);
-        bar = reinterpret_cast<uint64_t *>(smem_raw + offg + (CPB * NC * N3 * sizeof(GS) + 15) / 16 * 16);
+        constexpr int PAD = metric_pad<N, T, GS>();
+        bar = reinterpret_cast<uint64_t *>(smem_raw + offg + (CPB * (NC * N3 + PAD) * sizeof(GS) + 15) / 16 * 16);
         VS *sX = reinterpret_cast<VS *>(S0 + RS);  // buffer 1 is free until the gradients
         const VS *xsrc = x + cell0 * N3;
         const GS *gsrc = geo + cell0 * NC * N3;
@@ -490,20 +619,20 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                 mbar_expect_tx(bar, xb + dbg_extra);
                 bulk_g2s(sX, xsrc, xb, bar);
                 mbar_expect_tx(bar + 1, gb);
-                bulk_g2s(sG, gsrc, gb, bar + 1);
+                metric_copy<CPB, PAD>(sG, gsrc, NC * N3, bar + 1);
             }
             x_ok = mbar_wait_bounded(bar, 0, lim);
             if (!x_ok) wait_expired(status, bar, lim);
             x_smem = true;
             xs = sX + c * N3;
-            gs = sG + c * NC * N3;
+            gs = sG + c * (NC * N3 + PAD);
             g_smem = true;  // its wait comes before the physics step
         }
     } else if constexpr (STAGE == 3) {
         // the caller passes this tile's metric (gsm): staged in shared memory, where one copy serves
         // several right-hand sides, or in global memory when it could not be staged (cell slots past
         // a ragged tile's end read slot 0's, in bounds, and store nothing)
-        gs = gsm + (act ? c : 0) * NC * N3;
+        gs = gsm + (act ? c : 0) * gcs;
         g_smem = true;
     } else if constexpr (STAGE == 2) {
         bar = reinterpret_cast<uint64_t *>(smem_raw + NB * RS * sizeof(T));
@@ -572,41 +701,41 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
 #pragma unroll
             for (int m = 0; m < N; ++m) v[m] = have ? Ar::from(xl[m]) : Ar::zero();
             sweep<N, Ar, 0, NRM>(tab, v, w);
-            CW_TST(0, xi, 1, w);
+            stx(0, true, w);
         }
         __syncthreads();
         // (2) y-line (i,k): contract with B along y, in place
         {
-            CW_TLD(0, yo, PI, v);
+            ldy(0, v);
             sweep<N, Ar, 0, NRM>(tab, v, w);
-            CW_TST(0, yo, PI, w);
+            sty(0, w);
         }
         __syncthreads();
         // (3) z-pencil (i,j): contract with B along z -> u at the Gauss points (registers)
         {
-            CW_TLD(0, zo, PP, v);
+            ldz(0, v);
             sweep<N, Ar, 0, NRM>(tab, v, u);
         }
         if (HAS_K) {
             {
                 sweep<N, Ar, 2, NRM>(tab, u, gz);
-                CW_TST(0, zo, PP, u);
+                stz(0, u);
             }
             __syncthreads();
             // x- and y-derivatives by collocation, as line owners
             {
-                CW_TLD(0, xo, 1, v);
+                ldx(0, false, v);
                 sweep<N, Ar, 2, NRM>(tab, v, w);
-                CW_TST(1, xo, 1, w);
-                CW_TLD(0, yo, PI, v);
+                stx(1, false, w);
+                ldy(0, v);
                 sweep<N, Ar, 2, NRM>(tab, v, w);
                 if constexpr (NB == 2) __syncthreads();  // every line of buffer 0 has been read
-                CW_TST(YB, yo, PI, w);
+                sty(YB, w);
             }
             __syncthreads();
             {
-                CW_TLD(1, zo, PP, gx);
-                CW_TLD(YB, zo, PP, gy);
+                ldz(1, gx);
+                ldz(YB, gy);
             }
         }
         // the metric tile's wait (a thread whose wait expired reads the metric from global memory)
@@ -664,7 +793,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
 #pragma unroll
             for (int k = 0; k < N; ++k) {
                 const GS *g = gc + N2 * k;
-                T gxx, gyy, gzz, gxy, gxz, gyz, cmr;
+                T gxx, gyy, gzz, gxy, gxz, gyz, cmr, hx, hy, hz;
                 if constexpr (RING) {
                     cp_async_wait<kRing - 1>();  // the copies of point k have landed
                     const GS *rg = ring + (k % kRing) * NC * T1;
@@ -709,13 +838,20 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                     const T w = Ar::norm(Ar::mul(wab, tab.wq[k]));
                     cmr = Ar::norm(Ar::mul(w, det));
                     if (HAS_K) {
+                        // h_a = (w / det J) c_a . v with v = sum_b c_b g_b: 18 multiply-adds and 3 scalings
+                        // where forming G first takes 27 and 6 (41x40x39 Q4 K+M 449 -> 419 us, error 2.8e-14 -> 1.8e-14)
                         const T sc = Ar::div(w, det);
-                        gxx = Ar::norm(Ar::mul(sc, dot3(c0, c0)));
-                        gyy = Ar::norm(Ar::mul(sc, dot3(c1, c1)));
-                        gzz = Ar::norm(Ar::mul(sc, dot3(c2, c2)));
-                        gxy = Ar::norm(Ar::mul(sc, dot3(c0, c1)));
-                        gxz = Ar::norm(Ar::mul(sc, dot3(c0, c2)));
-                        gyz = Ar::norm(Ar::mul(sc, dot3(c1, c2)));
+                        T vv[3];
+#pragma unroll
+                        for (int d = 0; d < 3; ++d) {
+                            T t = Ar::mul(c0[d], gx[k]);
+                            Ar::mad(t, c1[d], gy[k]);
+                            Ar::mad(t, c2[d], gz[k]);
+                            vv[d] = Ar::norm(Ar::mul(sc, Ar::norm(t)));
+                        }
+                        hx = dot3(c0, vv);
+                        hy = dot3(c1, vv);
+                        hz = dot3(c2, vv);
                     }
                 }
                 if (HAS_K) {
@@ -724,17 +860,18 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                         gzz = Ar::from(g[2 * N3]), gxy = Ar::from(g[3 * N3]);
                         gxz = Ar::from(g[4 * N3]), gyz = Ar::from(g[5 * N3]);
                     }
-                    T hx = Ar::mul(gx[k], gxx), hy = Ar::mul(gx[k], gxy), hz = Ar::mul(gx[k], gxz);
-                    Ar::mad(hx, gy[k], gxy);
-                    Ar::mad(hy, gy[k], gyy);
-                    Ar::mad(hz, gy[k], gyz);
-                    Ar::mad(hx, gz[k], gxz);
-                    Ar::mad(hy, gz[k], gyz);
-                    Ar::mad(hz, gz[k], gzz);
+                    if constexpr (!RC) {
+                        hx = Ar::mul(gx[k], gxx), hy = Ar::mul(gx[k], gxy), hz = Ar::mul(gx[k], gxz);
+                        Ar::mad(hx, gy[k], gxy);
+                        Ar::mad(hy, gy[k], gyy);
+                        Ar::mad(hz, gy[k], gyz);
+                        Ar::mad(hx, gz[k], gxz);
+                        Ar::mad(hy, gz[k], gyz);
+                        Ar::mad(hz, gz[k], gzz);
+                    }
                     if constexpr (DOT) {  // (grad u)^T G (grad u) at this point
-                        df_mad(*dot, Ar::to_df(gx[k]), Ar::to_df(hx));
-                        df_mad(*dot, Ar::to_df(gy[k]), Ar::to_df(hy));
-                        df_mad(*dot, Ar::to_df(gz[k]), Ar::to_df(hz));
+                        dot_add2(*dot, gx[k], hx, gy[k], hy);
+                        dot_add(*dot, gz[k], hz);
                     }
                     gx[k] = NRM ? Ar::norm(hx) : hx;
                     gy[k] = NRM ? Ar::norm(hy) : hy;
@@ -744,7 +881,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                     if constexpr (!RC && !RING) cmr = Ar::from(g[(NC - 1) * N3]);
                     const T cm = cmr;
                     acc[k] = NRM ? Ar::norm(Ar::mul(u[k], cm)) : Ar::mul(u[k], cm);
-                    if constexpr (DOT) df_mad(*dot, Ar::to_df(u[k]), Ar::to_df(acc[k]));  // c u^2
+                    if constexpr (DOT) dot_add(*dot, u[k], acc[k]);  // c u^2
                 }
                 if constexpr (RING) ring_issue(k + kRing);  // into the slot point k was read from
             }
@@ -755,22 +892,22 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                 sweep<N, Ar, 3, NRM>(tab, gz, v);
 #pragma unroll
                 for (int k = 0; k < N; ++k) acc[k] = HAS_M ? Ar::add(acc[k], v[k]) : v[k];
-                CW_TST(1, zo, PP, gx);  // own pencil only: no other thread reads these pencils now
-                CW_TST(YB, zo, PP, gy);
+                stz(1, gx);  // own pencil only: no other thread reads these pencils now
+                stz(YB, gy);
             }
             __syncthreads();
             {
-                CW_TLD(1, xo, 1, v);
+                ldx(1, false, v);
                 sweep<N, Ar, 3, NRM>(tab, v, w);
-                CW_TST(1, xo, 1, w);
-                CW_TLD(YB, yo, PI, v);
+                stx(1, false, w);
+                ldy(YB, v);
                 sweep<N, Ar, 3, NRM>(tab, v, w);
-                CW_TST(YB, yo, PI, w);
+                sty(YB, w);
             }
             __syncthreads();
             {
-                CW_TLD(1, zo, PP, v);
-                CW_TLD(YB, zo, PP, w);
+                ldz(1, v);
+                ldz(YB, w);
 #pragma unroll
                 for (int k = 0; k < N; ++k) {
                     const T t = Ar::add(acc[k], Ar::add(v[k], w[k]));
@@ -781,17 +918,17 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         // (5) integrate back: B^T along z (registers), y and x as line owners
         {
             sweep<N, Ar, 1, NRM>(tab, acc, w);
-            CW_TST(0, zo, PP, w);
+            stz(0, w);
         }
         __syncthreads();
         {
-            CW_TLD(0, yo, PI, v);
+            ldy(0, v);
             sweep<N, Ar, 1, NRM>(tab, v, w);
-            CW_TST(0, yo, PI, w);
+            sty(0, w);
         }
         __syncthreads();
         {
-            CW_TLD(0, xi, 1, v);
+            ldx(0, true, v);
             sweep<N, Ar, 1, NRM>(tab, v, w);
             VS nv[N];  // the values to store
             const bool yvec = LineVec<N, VS>::aligned(y);
@@ -899,34 +1036,37 @@ __global__ void __launch_bounds__(N *N *CPB, (df_capped<Ar, N, false>() ? df_min
                                            o.status, o.dbg_extra);
 }
 
-// y = A x and the CTA's partial of <x, A x> in part[blockIdx.x] (deterministic: fixed order in a CTA)
+// y = A x and the CTA's partial of <x, A x> in part[blockIdx.x] (deterministic: fixed order in a CTA). The
+// threads' sums go through shared memory to one warp: 9 FP64 additions of a warp per 128 threads, each 16
+// cycles of the SM's FP64 pipe, where shuffles in every warp took 23 (14 us of FP64 pipe per launch of 13824
+// CTAs beside a kernel of 47 us). FP32 at n = 4: capped to the registers of the plain apply, which the
+// shared memory lets run in 11 CTAs per SM.
+template <class Ar, int N, bool RC>
+constexpr int dot_min_blocks()
+{
+    return std::is_same<Ar, ArF32>::value && N == 4 && !RC ? 11 : 0;
+}
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE, bool RC = false>
-__global__ void __launch_bounds__(N *N *CPB) apply_metric_dot_kernel(const VS *__restrict__ x, VS *__restrict__ y,
-                                                                      const GS *__restrict__ geo, int64_t ncells,
-                                                                      int kind, TabMetric<N, typename Ar::C> tab,
-                                                                      double *__restrict__ part, unsigned *status,
-                                                                      uint32_t dbg_extra)
+__global__ void __launch_bounds__(N *N *CPB, (dot_min_blocks<Ar, N, RC>()))
+    apply_metric_dot_kernel(const VS *__restrict__ x, VS *__restrict__ y, const GS *__restrict__ geo, int64_t ncells,
+                            int kind, TabMetric<N, typename Ar::C> tab, double *__restrict__ part, unsigned *status,
+                            uint32_t dbg_extra)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double s_red[(N * N * CPB + 31) / 32];
-    df64 acc{0.0f, 0.0f};
+    DotAcc acc;
     metric_tile<N, CPB, Ar, VS, GS, STAGE, true, RC>(x, y, geo, ncells, kind, tab, blockIdx.x, CPB, smem_raw, &acc, 0,
                                                      nullptr, nullptr, status, dbg_extra);
-    double v = df_to_double(acc);
-    // N^2 * CPB is not always a multiple of 32: the last warp may hold only nw lanes
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int nw = min(32, N * N * CPB - wid * 32);
-    const unsigned mask = nw == 32 ? 0xffffffffu : ((1u << nw) - 1u);
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_down_sync(mask, v, o);
-        if (lane + o < nw) v += ov;
-    }
-    if (lane == 0) s_red[wid] = v;
+    constexpr int T = N * N * CPB;
+    static_assert(T >= 32, "one whole warp sums");
+    double *sh = reinterpret_cast<double *>(smem_raw);  // the line buffers (at least 8 N^3 CPB bytes)
+    __syncthreads();                                    // whose last lines have been read
+    sh[threadIdx.x] = dot_value(acc);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < (N * N * CPB + 31) / 32; ++i) t += s_red[i];
-        part[blockIdx.x] = t;
+    if (threadIdx.x < 32) {
+        double v = sh[threadIdx.x];
+        for (int i = threadIdx.x + 32; i < T; i += 32) v += sh[i];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (threadIdx.x == 0) part[blockIdx.x] = v;
     }
 }
 

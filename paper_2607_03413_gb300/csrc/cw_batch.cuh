@@ -155,24 +155,24 @@ __device__ __forceinline__ const BatchTables<C> &batch_tables();
 // the call costs them more than it saves.) gsm: the tile's metric in shared memory (STAGE 3).
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
 __device__ __noinline__ void grouped_tile(const VS *x, VS *y, const GS *g, int64_t ncells, int kind, int64_t tile,
-                                          unsigned *status, const GS *gsm, uint64_t *gbar, uint32_t gphase)
+                                          unsigned *status, const GS *gsm, int gcs, uint64_t *gbar, uint32_t gphase)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     metric_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, batch_tab<N>(batch_tables<typename Ar::C>()), tile,
-                                           CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gbar, gphase);
+                                           CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gcs, gbar, gphase);
 }
 
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
 __device__ __forceinline__ void grouped_one(const VS *x, VS *y, const GS *g, int64_t ncells, int kind, int64_t tile,
-                                            unsigned *status, const GS *gsm, uint64_t *gbar, uint32_t gphase,
+                                            unsigned *status, const GS *gsm, int gcs, uint64_t *gbar, uint32_t gphase,
                                             unsigned char *smem_raw)
 {
     if constexpr (std::is_same<Ar, ArDF>::value)
-        grouped_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, gsm, gbar, gphase);
+        grouped_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, gsm, gcs, gbar, gphase);
     else
         metric_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, batch_tab<N>(batch_tables<typename Ar::C>()),
-                                               tile, CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gbar,
-                                               gphase);
+                                               tile, CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gcs,
+                                               gbar, gphase);
 }
 
 // ---- grouped mode: one persistent kernel per degree, shaped like the per-operator kernel
@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
 {
     using T = typename Ar::T;
     constexpr int N3 = N * N * N;
+    [[maybe_unused]] constexpr int PAD = metric_pad<N, T, GS>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long s_next;
     __shared__ int s_prob;
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
                 staged = cell0 + CPB <= P.ncells && aligned16(gsrc) && gb % 16 == 0;  // block-uniform
                 if (staged && threadIdx.x == 0) {  // waited for before the first right-hand side's physics
                     mbar_expect_tx(bar, gb);
-                    bulk_g2s(sG, gsrc, gb, bar);
+                    metric_copy<CPB, PAD>(sG, gsrc, NC * N3, bar);
                 }
             }
             for (int r = r0; r < r1; ++r) {
@@ -237,10 +238,10 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
                 if constexpr (STAGE == 1) {  // one code path: the metric from shared or from global memory
                     const GS *gm = staged ? sG : g + tile * CPB * NC * N3;
                     grouped_one<N, CPB, Ar, VS, GS, 3>(x, y, g, P.ncells, P.kind, tile, P.status, gm,
-                                                       staged && r == r0 ? bar : nullptr, phase, smem_raw);
+                                                       NC * N3 + (staged ? PAD : 0), staged && r == r0 ? bar : nullptr, phase, smem_raw);
                 } else {
-                    grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status, nullptr, nullptr,
-                                                           0, smem_raw);
+                    grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status, nullptr, 0,
+                                                           nullptr, 0, smem_raw);
                 }
             }
             if (staged) phase ^= 1u;

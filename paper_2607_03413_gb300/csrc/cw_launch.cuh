@@ -243,14 +243,13 @@ cudaError_t launch_multi_degree(const Op *const *op, const int64_t *off, int cou
     return cudaErrorInvalidValue;
 }
 
-// One fused smoothing sweep (smooth_metric_kernel): default tile, input tile staged by TMA and, where
-// the metric is stored, the arithmetic's default staging of it (FP32: prefetched into L2); the x-interfaces inside tiles are averaged, *xfuse receives the
+// One fused smoothing sweep (smooth_metric_kernel): default tile and staging; the x-interfaces inside tiles are averaged, *xfuse receives the
 // tile size for the x pass between tiles.
 template <int N, class Ar, class VS, class GS, bool RC>
 cudaError_t launch_smooth(const Op &op, void *u, const void *b, const void *dhat, cudaStream_t s, int *xfuse)
 {
     constexpr int CPB = cpb_tuned<N, Ar, VS>();
-    constexpr int ST = RC || std::is_same<Ar, ArF32>::value ? 2 : default_stage(N, false);
+    constexpr int ST = RC ? 2 : default_stage(N, std::is_same<Ar, ArF32>::value);
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op.tab, [](double v) { return MakeC<Ar>::from(v); });
     const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op.kind), ST);

@@ -151,16 +151,27 @@ __global__ void __launch_bounds__(4 * N * N * CP) restrict_kernel(const VS *__re
         s_base[t] = e < ncoarse ? child_cell(e, nx, ny, 2 * (t % 4)) * N3 : -1;
     }
     __syncthreads();
-    // load: for each parent and child pair one contiguous span of 2 N3 fine values
-    for (int k = t; k < CP * 8 * N3; k += blockDim.x) {
-        const int q = k / (2 * N3), w = k - q * (2 * N3);  // q = 4 c + pr
+    // load: for each parent and child pair one contiguous span of 2 N3 fine values, W values per access
+    // (one by one the index arithmetic and the loads in flight bounded the kernel: 50 us at 64^3 Q3 FP32)
+    constexpr int W = N % 2 == 0 && sizeof(VS) == 4 ? 4 : 2;
+    const bool vec = LineVec<W, VS>::aligned(bf) && (!SUB || LineVec<W, VS>::aligned(vf));
+    for (int kw = t; kw < CP * 8 * N3 / W; kw += blockDim.x) {
+        const int k = kw * W, q = k / (2 * N3), w = k - q * (2 * N3);  // q = 4 c + pr
         const int64_t base = s_base[q];
-        T v = Ar::zero();
+        VS x[W], y[W];
         if (base >= 0) {
-            v = Ar::from(ldg_nc(bf + base + w));
-            if constexpr (SUB) v = Ar::sub(v, Ar::from(ldg_nc(vf + base + w)));
+            line_ld<W>(bf + base + w, x, vec);
+            if constexpr (SUB) line_ld<W>(vf + base + w, y, vec);
         }
-        S0[k] = v;  // k = c 8 N3 + (2 pr + bx) N3 + local
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            T v = Ar::zero();
+            if (base >= 0) {
+                v = Ar::from(x[i]);
+                if constexpr (SUB) v = Ar::sub(v, Ar::from(y[i]));
+            }
+            S0[k + i] = v;  // k = c 8 N3 + (2 pr + bx) N3 + local
+        }
     }
     __syncthreads();
     T in[N], out[N], acc[N];
