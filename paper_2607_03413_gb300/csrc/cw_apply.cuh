@@ -542,6 +542,9 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         yo = yc * CS + (yr % N) + PP * (yr / N);
     }
 
+    // whole-line accesses of the input and output (LineVec) where they are wider than a value, but not at n = 6
+    // in 8-byte vectors, where they cost the double-float kernel 6 % (Q5, 128e6 values: 33.3 -> 31.2 G values/s)
+    constexpr bool WIDE = LineVec<N, VS>::WIDE && !(sizeof(VS) == 8 && N == 6);
     // load / store of a line of buffer R (0, 1, 2): x-line (own: the thread's own cell), y-line, z-pencil
     constexpr bool SW = tile_swizzled(N, sizeof(T), REMAP);
     using Z = TileSwz<N>;
@@ -688,10 +691,10 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
             bool have = act;
             if (x_smem) {  // a thread whose wait expired reads nothing staged
                 have = x_ok;
-                if (x_ok) LineVec<N, VS>::ld(xs + N * r, xl);
+                if (x_ok) line_ld<N>(xs + N * r, xl, WIDE);
             } else if (act) {
                 const VS *xg = x + cell * N3 + N * r;
-                if (LineVec<N, VS>::aligned(x)) {
+                if (WIDE && LineVec<N, VS>::aligned(x)) {
                     LineVec<N, VS>::ld_nc(xg, xl);
                 } else {
 #pragma unroll
@@ -931,7 +934,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
             ldx(0, true, v);
             sweep<N, Ar, 1, NRM>(tab, v, w);
             VS nv[N];  // the values to store
-            const bool yvec = LineVec<N, VS>::aligned(y);
+            const bool yvec = WIDE && LineVec<N, VS>::aligned(y);
             const int64_t o = (act ? cell : 0) * N3 + N * r;
 #pragma unroll
             for (int m = 0; m < N; ++m) Ar::to(nv[m], w[m]);
@@ -1106,18 +1109,10 @@ __global__ void __launch_bounds__(N *N *CPB) apply_affine_kernel(const VS *__res
     T v[N], P[N], Q[N];
     // x-line: P = M_x u, Q = K_x u
     {
-        VS xl[N];
-        if (act) {
-            const VS *xc = x + cell * N3 + N * r;
-            if (LineVec<N, VS>::aligned(x)) {
-                LineVec<N, VS>::ld_nc(xc, xl);
-            } else {
+        // (whole-line loads were 6-8 % slower here)
+        const VS *xc = x + (act ? cell : 0) * N3 + N * r;
 #pragma unroll
-                for (int m = 0; m < N; ++m) xl[m] = ldg_nc(xc + m);
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < N; ++m) v[m] = act ? Ar::from(xl[m]) : Ar::zero();
+        for (int m = 0; m < N; ++m) v[m] = act ? Ar::from(ldg_nc(xc + m)) : Ar::zero();
         contract<N, false, Ar>(tab.M, v, P);
         CW_STX(s0, P);
         if (HAS_K) {

@@ -4,8 +4,9 @@
 // Single mode: work items are (problem, chunk of tiles, right-hand side) with the right-hand side
 // fastest, so the R items of one chunk run at nearly the same time and its metric comes from HBM once
 // and from L2 for the other R-1. Grouped mode: items are (problem, chunk of tiles), and an item runs all
-// R right-hand sides through every tile with the tile's metric staged in shared memory once. A chunk holds about kItemValues cell-wise values, enough work to hide the
-// per-item cost (an atomicAdd on the global counter, a search of the problem table). Each CTA
+// R right-hand sides through every tile with the tile's metric staged in shared memory once. A chunk holds at
+// most about kItemValues cell-wise values, enough work to hide the per-item cost (an atomicAdd on the global
+// counter, a look-up in the problem table), and fewer where the SMs would run out of items (item_tiles). Each CTA
 // (128 threads) fetches the number of its next item while it works on the current one; an item
 // number past the end ends the CTA (no spinning). The tile size is chosen per degree: the largest
 // number of cells whose N*N threads fit in the CTA, or half of it (the remaining cell slots compute
@@ -266,7 +267,7 @@ inline int degree_cpb(int n, int alt, bool f32)
 template <class T>
 inline size_t batch_smem_bytes(int n)
 {
-    switch (n) {  // the three line buffers of metric_tile in this mode (lines in thread order)
+    switch (n) {  // the line buffers of metric_tile in this mode (lines in thread order)
     case 2: return metric_smem_bytes<2, batch_slots(2), T, float, false>(0, 0);
     case 3: return metric_smem_bytes<3, batch_slots(3), T, float, false>(0, 0);
     case 4: return metric_smem_bytes<4, batch_slots(4), T, float, false>(0, 0);

@@ -601,7 +601,7 @@ static bool apply_dot_ok(const Op &op, int ak)
     const bool f32 = prec_f32_arith(op.prec);
     if (op.geom == CW_GEOM_METRIC ? op.stage != 1 && op.stage != default_stage(op.n, f32) : op.geom != CW_GEOM_RECOMPUTE)
         return false;
-    if (op.cpb != 0 && !default_cells(op.n, f32, true)) return false;  // not the default tile
+    if (op.cpb != 0 && !(op.geom == CW_GEOM_METRIC && default_cells(op.n, f32, op.prec == CW_PREC_F32))) return false;  // not the default tile
     return op.prec == CW_PREC_F64 || op.prec == CW_PREC_F32 || op.prec == CW_PREC_F32_BF16G;
 }
 

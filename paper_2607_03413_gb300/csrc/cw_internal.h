@@ -36,9 +36,11 @@ __host__ __device__ constexpr int tile_cells(int n, bool f32)
 // 51^3 Q5 985 / 866, but 99^3 Q2 472 / 531, 78^3 Q3 526 / 547, 64^3 Q4 779 / 795, 42^3 Q6 787 / 846,
 // 35^3 Q7 694 / 735.
 __host__ __device__ constexpr int default_stage(int n, bool f32) { return !f32 && n == 6 ? 2 : 1; }
-// Whether an operator starts with the alternative tile (half the default): FP32 vectors at n = 7, where
-// 8 cells are 2 CTAs per SM (42^3 Q6 Laplace 175 us with 4 cells, 281 with 8; BF16 182 with 8, 216 with 4).
-__host__ __device__ constexpr bool default_cells(int n, bool f32, bool vec4) { return f32 && n == 7 && vec4; }
+// Whether a stored-metric operator starts with the alternative tile (half the default): FP32 vectors and
+// metric (g4) at n = 7, where 8 cells are 2 CTAs per SM (42^3 Q6 Laplace 175 us with 4 cells, 281 with 8; BF16
+// 182 with 8, 216 with 4). With a BF16 metric 4 cells would not do: their tile of 7 or 1 components is no
+// multiple of the 16 bytes that a bulk copy moves (31x32x28 Q6 K+M assembled 173 us instead of 106).
+__host__ __device__ constexpr bool default_cells(int n, bool f32, bool g4) { return f32 && n == 7 && g4; }
 
 // whether a precision computes in FP32 arithmetic (its kernels use the FP32 tile sizes)
 __host__ __device__ inline bool prec_f32_arith(int prec)

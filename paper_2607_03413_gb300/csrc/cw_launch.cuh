@@ -111,10 +111,11 @@ constexpr int cpb_alt()
 }
 
 // the tile an operator starts with (default_cells): the default, or the alternative where it is faster
-template <int N, class Ar, class VS>
+template <int N, class Ar, class VS, class GS, bool RC>
 constexpr int cpb_tuned()
 {
-    return default_cells(N, std::is_same<Ar, ArF32>::value, sizeof(VS) == 4) ? cpb_alt<N, Ar>() : cpb_default<N, Ar>();
+    return !RC && default_cells(N, std::is_same<Ar, ArF32>::value, sizeof(VS) == 4 && sizeof(GS) == 4) ? cpb_alt<N, Ar>()
+                                                                                                     : cpb_default<N, Ar>();
 }
 
 template <class K>
@@ -204,7 +205,7 @@ template <int N, class Ar, class VS, class GS>
 cudaError_t launch_multi(const Op *const *op, const int64_t *off, int count, const void *x, void *y, int *xtile,
                          cudaStream_t s)
 {
-    constexpr int CPB = cpb_tuned<N, Ar, VS>(), ST = default_stage(N, std::is_same<Ar, ArF32>::value);
+    constexpr int CPB = cpb_tuned<N, Ar, VS, GS, false>(), ST = default_stage(N, std::is_same<Ar, ArF32>::value);
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op[0]->tab, [](double v) { return MakeC<Ar>::from(v); });
     const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op[0]->kind), ST);
@@ -248,7 +249,7 @@ cudaError_t launch_multi_degree(const Op *const *op, const int64_t *off, int cou
 template <int N, class Ar, class VS, class GS, bool RC>
 cudaError_t launch_smooth(const Op &op, void *u, const void *b, const void *dhat, cudaStream_t s, int *xfuse)
 {
-    constexpr int CPB = cpb_tuned<N, Ar, VS>();
+    constexpr int CPB = cpb_tuned<N, Ar, VS, GS, RC>();
     constexpr int ST = RC ? 2 : default_stage(N, std::is_same<Ar, ArF32>::value);
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op.tab, [](double v) { return MakeC<Ar>::from(v); });
@@ -290,7 +291,7 @@ cudaError_t launch_smooth_degree(const Op &op, void *u, const void *b, const voi
 template <int N, class Ar, class VS, class GS, bool RC = false>
 cudaError_t launch_metric_dot(const Op &op, const void *x, void *y, double *part, int64_t *nblocks, cudaStream_t s)
 {
-    constexpr int CPB = cpb_tuned<N, Ar, VS>(), ST = RC ? 2 : default_stage(N, std::is_same<Ar, ArF32>::value);
+    constexpr int CPB = cpb_tuned<N, Ar, VS, GS, RC>(), ST = RC ? 2 : default_stage(N, std::is_same<Ar, ArF32>::value);
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op.tab, [](double v) { return MakeC<Ar>::from(v); });
     const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op.kind), ST);

@@ -17,6 +17,7 @@ struct LineVec {
     static constexpr int BYTES = N * (int)sizeof(V);
     static constexpr int VB = BYTES % 16 == 0 ? 16 : BYTES % 8 == 0 ? 8 : BYTES % 4 == 0 ? 4 : 2;
     static constexpr int NW = BYTES / VB;
+    static constexpr bool WIDE = VB > (int)sizeof(V);  // else (odd N) value by value is all there is
     using W = std::conditional_t<VB == 16, uint4,
                                  std::conditional_t<VB == 8, uint2, std::conditional_t<VB == 4, uint32_t, uint16_t>>>;
     static_assert(VB >= (int)sizeof(V), "a line is a whole number of accesses");
@@ -53,7 +54,7 @@ struct LineVec {
 template <int N, class V>
 __device__ __forceinline__ void line_ld(const V *p, V (&v)[N], bool vec)
 {
-    if (vec) {
+    if (LineVec<N, V>::WIDE && vec) {
         LineVec<N, V>::ld(p, v);
     } else {
 #pragma unroll
@@ -63,7 +64,7 @@ __device__ __forceinline__ void line_ld(const V *p, V (&v)[N], bool vec)
 template <int N, class V>
 __device__ __forceinline__ void line_st(V *p, const V (&v)[N], bool vec)
 {
-    if (vec) {
+    if (LineVec<N, V>::WIDE && vec) {
         LineVec<N, V>::st(p, v);
     } else {
 #pragma unroll
