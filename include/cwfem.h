@@ -190,8 +190,7 @@ int64_t cw_op_device_bytes(cw_op op);
  * the two choices cw_op_get_variant reports -- and stage: 0 direct loads; 1 each CTA's input and
  * metric tiles moved into shared memory with bulk asynchronous copies (TMA) at kernel entry; 2 the
  * input tile by TMA and the metric tile prefetched into L2 by a bulk prefetch (less shared memory,
- * more CTAs per SM), from where CW_PREC_F64 threads copy their entries two quadrature points ahead. An
- * operator starts with the choice that measured fastest for its degree and precision. Results do not depend on the variant beyond rounding order. CW_PREC_F64_NATIVE has only
+ * more CTAs per SM). An operator starts with the choice that measured fastest for its degree and precision. Results do not depend on the variant beyond rounding order. CW_PREC_F64_NATIVE has only
  * the default variant (CW_ERR_UNSUPPORTED otherwise). CW_GEOM_RECOMPUTE operators use the default
  * cells per CTA (another choice gives CW_ERR_UNSUPPORTED); stages 1 and 2 both stage the input
  * tile by TMA there (there is no metric tile).

@@ -426,15 +426,6 @@ constexpr int line_buffers()
     return sizeof(T) == 8 ? 2 : 3;
 }
 
-// Stage 2 in double-float arithmetic: each thread copies the metric entries of its own pencil into a
-// private ring of kRing points in shared memory with 8-byte cp.async, kRing points ahead of their use.
-constexpr int kRing = 2;
-template <class Ar, int STAGE, bool RC>
-constexpr bool metric_ring()
-{
-    return std::is_same<Ar, ArDF>::value && STAGE == 2 && !RC;
-}
-
 // Elements between the staged metrics of two cells beyond their own: at n = 4 in FP32 arithmetic the two cells
 // of a warp read the same banks (a cell's metric is a multiple of 32 words), so each cell gets 64 bytes more
 // and a bulk copy of its own.
@@ -459,7 +450,7 @@ template <int N, int CPB, class T, class GS, bool REMAP = true>
 __host__ __device__ constexpr size_t metric_smem_bytes(int nc, int stage)
 {
     constexpr size_t lb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), REMAP>::RS * sizeof(T);  // a multiple of 16
-    return stage == 1 ? lb + (CPB * (nc * N * N * N + metric_pad<N, T, GS>()) * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 + (std::is_same<T, df64>::value ? kRing * nc * N * N * CPB * sizeof(GS) : 0) : lb;
+    return stage == 1 ? lb + (CPB * (nc * N * N * N + metric_pad<N, T, GS>()) * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 : lb;
 }
 
 // One tile of `cpt` consecutive cells starting at cell tile*cpt, worked by CPB cell slots of N*N
@@ -662,27 +653,6 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         }
     }
 
-    // RING: this thread's ring of the metric entries of its next kRing points
-    constexpr bool RING = metric_ring<Ar, STAGE, RC>();
-    constexpr int T1 = N2 * CPB;
-    [[maybe_unused]] GS *ring = reinterpret_cast<GS *>(smem_raw + NB * RS * sizeof(T) + 16) + t;
-    [[maybe_unused]] const GS *gring = geo + (act ? cell : 0) * NC * N3 + r;
-    auto ring_issue = [&](int k) {
-        if (k < N) {
-            GS *d = ring + (k % kRing) * NC * T1;
-            const GS *g = gring + N2 * k;
-            if (HAS_K) {
-#pragma unroll
-                for (int i = 0; i < 6; ++i) cp_async8(d + i * T1, g + i * N3);
-            }
-            if (HAS_M) cp_async8(d + (NC - 1) * T1, g + (NC - 1) * N3);
-        }
-        cp_async_commit();  // one group per point, empty past the end
-    };
-    if constexpr (RING) {
-#pragma unroll
-        for (int k = 0; k < kRing; ++k) ring_issue(k);
-    }
     {
         T v[N], w[N], u[N], acc[N], gx[N], gy[N], gz[N];
         // (1) x-line (j,k) = (ra, rb): N contiguous values of the cell, contracted with B along x
@@ -797,15 +767,6 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
             for (int k = 0; k < N; ++k) {
                 const GS *g = gc + N2 * k;
                 T gxx, gyy, gzz, gxy, gxz, gyz, cmr, hx, hy, hz;
-                if constexpr (RING) {
-                    cp_async_wait<kRing - 1>();  // the copies of point k have landed
-                    const GS *rg = ring + (k % kRing) * NC * T1;
-                    if (HAS_K) {
-                        gxx = Ar::from(rg[0 * T1]), gyy = Ar::from(rg[1 * T1]), gzz = Ar::from(rg[2 * T1]);
-                        gxy = Ar::from(rg[3 * T1]), gxz = Ar::from(rg[4 * T1]), gyz = Ar::from(rg[5 * T1]);
-                    }
-                    if (HAS_M) cmr = Ar::from(rg[(NC - 1) * T1]);
-                }
                 if constexpr (RC) {
                     const T zeta = tab.xq[k];
                     T jx[3], jy[3];
@@ -858,7 +819,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                     }
                 }
                 if (HAS_K) {
-                    if constexpr (!RC && !RING) {
+                    if constexpr (!RC) {
                         gxx = Ar::from(g[0 * N3]), gyy = Ar::from(g[1 * N3]);
                         gzz = Ar::from(g[2 * N3]), gxy = Ar::from(g[3 * N3]);
                         gxz = Ar::from(g[4 * N3]), gyz = Ar::from(g[5 * N3]);
@@ -881,12 +842,11 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                     gz[k] = NRM ? Ar::norm(hz) : hz;
                 }
                 if (HAS_M) {
-                    if constexpr (!RC && !RING) cmr = Ar::from(g[(NC - 1) * N3]);
+                    if constexpr (!RC) cmr = Ar::from(g[(NC - 1) * N3]);
                     const T cm = cmr;
                     acc[k] = NRM ? Ar::norm(Ar::mul(u[k], cm)) : Ar::mul(u[k], cm);
                     if constexpr (DOT) dot_add(*dot, u[k], acc[k]);  // c u^2
                 }
-                if constexpr (RING) ring_issue(k + kRing);  // into the slot point k was read from
             }
         }
         if (HAS_K) {

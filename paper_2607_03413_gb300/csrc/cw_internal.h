@@ -31,11 +31,11 @@ __host__ __device__ constexpr int tile_cells(int n, bool f32)
 }
 
 // Staging mode a stored-metric operator starts with (op.stage). FP32 arithmetic: 1 (input and metric
-// tiles by TMA). Double-float: 1, but 2 (each thread's metric entries two points ahead by 8-byte
-// cp.async) at n = 6, where the staged metric leaves 3 CTAs of 4.5 warps per SM. Laplace, mode 1 / 2 us:
-// 51^3 Q5 985 / 866, but 99^3 Q2 472 / 531, 78^3 Q3 526 / 547, 64^3 Q4 779 / 795, 42^3 Q6 787 / 846,
-// 35^3 Q7 694 / 735.
-__host__ __device__ constexpr int default_stage(int n, bool f32) { return !f32 && n == 6 ? 2 : 1; }
+// tiles by TMA). Double-float: 1, but 2 (metric prefetched into L2 and loaded in place) at n = 6 and 8, where
+// the staged metric's shared memory leaves 3 CTAs of 4 or 5 warps per SM. Laplace, mode 1 / 2 us: 51^3 Q5
+// 979 / 878, 35^3 Q7 699 / 684, but 99^3 Q2 471 / 502, 78^3 Q3 526 / 531, 64^3 Q4 K+M 790 / 798, 42^3 Q6
+// 785 / 838.
+__host__ __device__ constexpr int default_stage(int n, bool f32) { return !f32 && (n == 6 || n == 8) ? 2 : 1; }
 // Whether a stored-metric operator starts with the alternative tile (half the default): FP32 vectors and
 // metric (g4) at n = 7, where 8 cells are 2 CTAs per SM (42^3 Q6 Laplace 175 us with 4 cells, 281 with 8; BF16
 // 182 with 8, 216 with 4). With a BF16 metric 4 cells would not do: their tile of 7 or 1 components is no
