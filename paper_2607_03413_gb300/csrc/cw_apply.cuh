@@ -414,8 +414,10 @@ __host__ __device__ constexpr int metric_ncomp(int kind) { return kind == 1 ? 6 
 // TMA, metric tile prefetched into L2 by a bulk prefetch (a third of the shared memory of mode 1,
 // so more CTAs per SM), then read with direct loads; 3: the metric tile in shared memory or on its way
 // there (staged by the caller for several right-hand sides: gsm, gcs elements per cell; gbar != nullptr: the
-// copy completes
-// phase gphase of *gbar, waited for before the physics step), x read directly.
+// copy completes phase gphase of *gbar, waited for before the physics step), x read directly.
+// A persistent caller, whose CTAs work on one tile after another, runs STAGE 2 on a barrier of its own: an
+// mbarrier must not be initialised again while it is live, so the caller initialises *gbar once, passes the
+// phase the next staged tile completes (gphase) and counts the staged tiles with x_tile_stageable.
 // Line buffers of metric_tile: three for 4-byte elements; two for 8-byte ones (double-float and FP64
 // arithmetic), whose y-derivatives go back into buffer 0 after one more barrier: with the metric staged
 // a CTA then needs 72 instead of 80 bytes of shared memory per value (K+M), which is one more CTA per SM
@@ -451,6 +453,13 @@ __host__ __device__ constexpr size_t metric_smem_bytes(int nc, int stage)
 {
     constexpr size_t lb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), REMAP>::RS * sizeof(T);  // a multiple of 16
     return stage == 1 ? lb + (CPB * (nc * N * N * N + metric_pad<N, T, GS>()) * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 : lb;
+}
+
+// whether a whole tile of CPB cells can be moved by one bulk copy from vector x (16-byte alignment and size)
+template <int N, int CPB, class VS>
+__device__ __forceinline__ bool x_tile_stageable(const VS *x, int64_t cell0, int64_t ncells)
+{
+    return cell0 + CPB <= ncells && (CPB * N * N * N * sizeof(VS)) % 16 == 0 && aligned16(x + cell0 * (N * N * N));
 }
 
 // One tile of `cpt` consecutive cells starting at cell tile*cpt, worked by CPB cell slots of N*N
@@ -636,18 +645,23 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         const int gpc = RC ? GV : NC * N3;
         const GS *gsrc = geo + cell0 * gpc;
         const uint32_t xb = CPB * N3 * sizeof(VS), gb = CPB * gpc * sizeof(GS);
+        static_assert(RS * sizeof(T) % 16 == 0, "the staged input tile starts on a 16-byte boundary");
         const bool full = cell0 + CPB <= ncells;
-        const bool ok = full && aligned16(xsrc) && aligned16(sX) && (xb % 16 == 0);
+        const bool ok = x_tile_stageable<N, CPB>(x, cell0, ncells);
         if (t == 0 && full && aligned16(gsrc) && (gb % 16 == 0)) bulk_prefetch_l2(gsrc, gb);
         if (ok) {  // block-uniform
-            if (t == 0) mbar_init(bar, 1);
-            __syncthreads();
+            if (!gbar) {  // block-uniform
+                if (t == 0) mbar_init(bar, 1);
+                __syncthreads();
+            } else {
+                bar = gbar;
+            }
             if (t == 0) {
                 mbar_expect_tx(bar, xb + dbg_extra);
                 bulk_g2s(sX, xsrc, xb, bar);
             }
-            x_ok = mbar_wait_bounded(bar, 0, lim);
-            if (!x_ok) wait_expired(status, bar, lim);
+            x_ok = mbar_wait_bounded(bar, gphase, lim);
+            if (!x_ok) wait_expired(status, bar, lim, gphase);
             x_smem = true;
             xs = sX + c * N3;
         }

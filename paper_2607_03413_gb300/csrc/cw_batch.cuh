@@ -193,13 +193,13 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long s_next;
     __shared__ int s_prob;
-    // STAGE 1 layout: [line buffers][mbarrier, 16 B][metric tile]
+    // STAGE 1 layout: [line buffers][mbarrier, 16 B][metric tile]; STAGE 2: [line buffers][mbarrier]
     const size_t offb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), true>::RS * sizeof(T);  // a multiple of 16
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + offb);
     GS *sG = reinterpret_cast<GS *>(smem_raw + offb + 16);
-    [[maybe_unused]] uint32_t phase = 0;  // of the metric tile's barrier
+    [[maybe_unused]] uint32_t phase = 0;  // of the barrier: flips with every staged tile
     if (threadIdx.x == 0) {
-        if constexpr (STAGE == 1) mbar_init(bar, 1);
+        if constexpr (STAGE != 0) mbar_init(bar, 1);  // once: it is live to the end of the CTA
         s_next = static_cast<long long>(atomicAdd(counter, 1ull));
     }
     for (;;) {
@@ -241,8 +241,11 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
                     grouped_one<N, CPB, Ar, VS, GS, 3>(x, y, g, P.ncells, P.kind, tile, P.status, gm,
                                                        NC * N3 + (staged ? PAD : 0), staged && r == r0 ? bar : nullptr, phase, smem_raw);
                 } else {
+                    if constexpr (STAGE == 2) staged = x_tile_stageable<N, CPB>(x, tile * CPB, P.ncells);
                     grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status, nullptr, 0,
-                                                           nullptr, 0, smem_raw);
+                                                           STAGE == 2 ? bar : nullptr, phase, smem_raw);
+                    // the next staged tile is copied over this one's line buffers, behind a barrier
+                    if constexpr (STAGE == 2) fence_async_shared();
                 }
             }
             if (staged) phase ^= 1u;

@@ -37,6 +37,11 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
+// Orders the calling thread's ordinary accesses to shared memory before bulk copies into it that a thread
+// issues behind the next barrier (ordinary accesses and bulk copies are different proxies, which a barrier
+// alone does not order). For kernels that stage a tile into memory an earlier tile used.
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // bulk prefetch of a global range into L2 (no shared memory, no completion to wait for)
 __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes)
 {
