@@ -223,7 +223,8 @@ cw_status cw_op_check(cw_op op, void *stream);
  * operator's kernels then arm the barrier of each staged input tile with 16 bytes more than the copy
  * delivers, so the copy lands but the barrier phase can never complete, the (shortened) bounded wait
  * runs out and the tile is abandoned and reported as above. Tiles read without staging (stage 0, a
- * ragged last tile) are not affected. Not for production use.
+ * ragged last tile) are not affected. A batch takes the state its operators have when it is created or its
+ * mode or a variant is set; its staging mode 1 arms the metric tiles' barrier. Not for production use.
  */
 cw_status cw_op_inject_stall(cw_op op, int on);
 

@@ -1515,7 +1515,7 @@ cw_status cw_op_inject_stall(cw_op oh, int on)
 {
     Op *op = reinterpret_cast<Op *>(oh);
     if (!op) return fail(CW_ERR_ARG, "cw_op_inject_stall: NULL handle");
-    op->dbg_tma_extra = on ? 16u : 0u;
+    op->dbg_tma_extra = on ? kStallBytes : 0u;
     op_generation_bump();
     return CW_OK;
 }

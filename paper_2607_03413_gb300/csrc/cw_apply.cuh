@@ -413,11 +413,11 @@ __host__ __device__ constexpr int metric_ncomp(int kind) { return kind == 1 ? 6 
 // STAGE 0: direct loads; 1: x and metric tiles staged in shared memory by TMA; 2: x tile staged by
 // TMA, metric tile prefetched into L2 by a bulk prefetch (a third of the shared memory of mode 1,
 // so more CTAs per SM), then read with direct loads; 3: the metric tile in shared memory or on its way
-// there (staged by the caller for several right-hand sides: gsm, gcs elements per cell; gbar != nullptr: the
-// copy completes phase gphase of *gbar, waited for before the physics step), x read directly.
-// A persistent caller, whose CTAs work on one tile after another, runs STAGE 2 on a barrier of its own: an
-// mbarrier must not be initialised again while it is live, so the caller initialises *gbar once, passes the
-// phase the next staged tile completes (gphase) and counts the staged tiles with x_tile_stageable.
+// there (staged by the caller for several right-hand sides: gsm, gcs elements per cell; pb != nullptr: its copy
+// completes a phase of *pb, waited for before the physics step), x read directly.
+// PERSIST: the caller's CTAs work on one tile after another, on a barrier of their own (pb): an mbarrier must not
+// be initialised again while it is live, so the caller initialises it once and passes each tile's state (st);
+// in STAGE 2 pb is null for a tile that is not staged.
 // Line buffers of metric_tile: three for 4-byte elements; two for 8-byte ones (double-float and FP64
 // arithmetic), whose y-derivatives go back into buffer 0 after one more barrier: with the metric staged
 // a CTA then needs 72 instead of 80 bytes of shared memory per value (K+M), which is one more CTA per SM
@@ -484,10 +484,35 @@ __device__ __forceinline__ bool x_tile_stageable(const VS *x, int64_t cell0, int
 // reaches memory.
 // An expired wait for a staged copy: record it in the device status word and wait once more (bounded)
 // so that the copy is not left in flight. Out of line: the common path carries none of it.
-static __device__ __noinline__ void wait_expired(unsigned *status, uint64_t *bar, uint32_t lim, uint32_t phase = 0)
+static __device__ __noinline__ void wait_expired(unsigned *status, uint64_t *bar, uint32_t lim)
 {
     if (status) atomicOr(status, kDevStatusTimeout);
-    mbar_wait_bounded(bar, phase, lim);
+    mbar_wait_bounded(bar, 0, lim);
+}
+// The same in a persistent CTA: a wait of some length continues here, up to the limit unless it is an injected
+// stall; an expired one is recorded for the CTA's next tiles too.
+__device__ __forceinline__ bool stage_wait_long(unsigned *status, StageBar *pb, unsigned st)
+{
+    const uint32_t phase = st & kTilePhase ? 1u : 0u;
+    if (!(st & kTileStalled) && mbar_wait_bounded(&pb->bar, phase, kWaitLimit)) return true;
+    if (status) atomicOr(status, kDevStatusTimeout);
+    atomicOr(&pb->expired, 1u);
+    mbar_wait_bounded(&pb->bar, phase, st & kTileStalled ? kWaitLimitInjected : kWaitLimit);
+    return false;
+}
+static __device__ __noinline__ bool stage_wait_long_call(unsigned *status, StageBar *pb, unsigned st)
+{
+    return stage_wait_long(status, pb, st);
+}
+// Whether the copy behind a persistent CTA's barrier has arrived (bounded wait). INL: the double-float tile is a
+// function of its own, in the middle of which a call costs registers (n = 6: 128 instead of 103); in the FP32
+// body, inlined into the persistent loop, the code itself does (n = 8: 96 instead of 80).
+template <bool INL>
+__device__ __forceinline__ bool stage_wait(unsigned *status, StageBar *pb, unsigned st)
+{
+    if (mbar_wait_bounded(&pb->bar, st & kTilePhase ? 1u : 0u, kWaitLimitInjected)) return true;
+    if constexpr (INL) return stage_wait_long(status, pb, st);
+    else return stage_wait_long_call(status, pb, st);
 }
 
 // Staged tiles and their waits: every wait for a bulk copy is bounded. A thread whose wait expired
@@ -496,20 +521,22 @@ static __device__ __noinline__ void wait_expired(unsigned *status, uint64_t *bar
 // CW_ERR_TIMEOUT by the next checking call: the outputs of that call are then undefined), and waits
 // once more (bounded) so that the copy is not left in flight. Nothing runs on the common path beyond
 // the wait itself: deciding the tile's fate block-wide (an early exit, or a flag read before the
-// stores) made the common path 2-6 % slower in measurement. dbg_extra > 0 (fault injection for tests)
-// arms the input tile's barrier with dbg_extra bytes more than the copy delivers, so that its phase
-// can never complete and the (then short) bounded wait runs out.
+// stores) made the common path 2-6 % slower in measurement. A persistent CTA, which has a barrier between its
+// tiles and right-hand sides anyway, does decide block-wide there (StageBar::expired). dbg_extra > 0 (fault
+// injection for tests) arms the input tile's barrier with dbg_extra bytes more than the copy delivers, so that
+// its phase can never complete and the (then short) bounded wait runs out.
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE, bool DOT = false, bool RC = false,
-          bool SMOOTH = false, bool REMAP = true>
+          bool SMOOTH = false, bool REMAP = true, bool PERSIST = false>
 __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__restrict__ geo,
                                             int64_t ncells, int kind, const TabMetric<N, typename Ar::C> &tab,
                                             int64_t tile, int cpt, unsigned char *smem_raw, DotAcc *dot = nullptr,
                                             int asm_nx = 0, const VS *sb = nullptr, const VS *sd = nullptr,
                                             unsigned *status = nullptr, uint32_t dbg_extra = 0,
-                                            const GS *gsm = nullptr, int gcs = 0, uint64_t *gbar = nullptr,
-                                            uint32_t gphase = 0)
+                                            StageBar *pb = nullptr, unsigned st = 0,
+                                            const GS *gsm = nullptr, int gcs = 0)
 {
     static_assert(!(RC && STAGE == 1), "recomputed geometry has no metric tile to stage");
+    static_assert(PERSIST ? STAGE != 1 : STAGE != 3, "staging mode 3 is that of persistent callers");
     // Double-float renormalisation of the intermediate values: kept where the operator serves the
     // solver (DOT), whose attainable accuracy depends on it (at 128^3 Q3 the double-float CG took
     // 1351 instead of 1026 iterations without it); skipped in the plain apply (5 % faster there,
@@ -600,7 +627,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
     const VS *xs = nullptr;
     const GS *gs = nullptr;
     uint64_t *bar = nullptr;
-    const uint32_t lim = dbg_extra ? kWaitLimitInjected : kWaitLimit;
+    [[maybe_unused]] const uint32_t lim = dbg_extra ? kWaitLimitInjected : kWaitLimit;
     if constexpr (STAGE == 1) {
         const size_t offg = NB * RS * sizeof(T);
         GS *sG = reinterpret_cast<GS *>(smem_raw + offg);
@@ -647,21 +674,25 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         const uint32_t xb = CPB * N3 * sizeof(VS), gb = CPB * gpc * sizeof(GS);
         static_assert(RS * sizeof(T) % 16 == 0, "the staged input tile starts on a 16-byte boundary");
         const bool full = cell0 + CPB <= ncells;
-        const bool ok = x_tile_stageable<N, CPB>(x, cell0, ncells);
+        const bool ok = PERSIST ? pb != nullptr : x_tile_stageable<N, CPB>(x, cell0, ncells);
         if (t == 0 && full && aligned16(gsrc) && (gb % 16 == 0)) bulk_prefetch_l2(gsrc, gb);
         if (ok) {  // block-uniform
-            if (!gbar) {  // block-uniform
+            if constexpr (PERSIST) {
+                bar = &pb->bar;
+            } else {
                 if (t == 0) mbar_init(bar, 1);
                 __syncthreads();
-            } else {
-                bar = gbar;
             }
             if (t == 0) {
-                mbar_expect_tx(bar, xb + dbg_extra);
+                mbar_expect_tx(bar, xb + (PERSIST ? (st & kTileStalled ? kStallBytes : 0u) : dbg_extra));
                 bulk_g2s(sX, xsrc, xb, bar);
             }
-            x_ok = mbar_wait_bounded(bar, gphase, lim);
-            if (!x_ok) wait_expired(status, bar, lim, gphase);
+            if constexpr (PERSIST) {
+                x_ok = stage_wait<std::is_same<Ar, ArDF>::value>(status, pb, st);
+            } else {
+                x_ok = mbar_wait_bounded(bar, 0, lim);
+                if (!x_ok) wait_expired(status, bar, lim);
+            }
             x_smem = true;
             xs = sX + c * N3;
         }
@@ -733,10 +764,8 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                 if (!g_ok) wait_expired(status, bar + 1, lim);
             }
         } else if constexpr (STAGE == 3) {
-            if (gbar) {  // block-uniform
-                g_ok = mbar_wait_bounded(gbar, gphase, lim);
-                if (!g_ok) wait_expired(status, gbar, lim, gphase);
-            }
+            if (pb)  // block-uniform
+                g_ok = stage_wait<std::is_same<Ar, ArDF>::value>(status, pb, st);
         }
         // (4) quadrature-point physics on the owned pencil, qp = (ra, rb, k)
         {

@@ -84,6 +84,7 @@ static cw_status batch_rebuild(Batch &b)
         P.y = b.y[i];
         P.geo = o.d_geo;
         P.status = o.d_status;
+        P.stall = o.dbg_tma_extra != 0;
         P.ncells = o.E;
         P.stride = o.L;
         P.n = o.n;

@@ -52,7 +52,8 @@ struct BatchProb {
     int64_t item0;      // first work item of this problem (items: chunk * nrhs + rhs)
     int64_t ntiles;     // tiles of cpt cells
     unsigned *status;   // the operator's device status word (an expired bounded wait is recorded there)
-    int n, kind, nrhs, cpt, tpi;  // tpi: tiles per chunk
+    short n, stall;  // stall: the operator's injected stall (tests of the failure report)
+    int kind, nrhs, cpt, tpi;  // tpi: tiles per chunk
 };
 
 template <class C>
@@ -153,27 +154,34 @@ __device__ __forceinline__ const BatchTables<C> &batch_tables();
 // persistent item loop, its 1D tables (loop-invariant, two floats per entry) were hoisted into
 // registers, which took the kernel from ~80 to 128-166 registers; out of line every table entry
 // stays an immediate constant-bank operand, as in the per-operator kernel. (FP32 bodies stay inline:
-// the call costs them more than it saves.) gsm: the tile's metric in shared memory (STAGE 3).
+// the call costs them more than it saves.) pb, st, gsm, gcs: the tile's barrier and metric (see metric_tile).
+template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
+__device__ __forceinline__ void grouped_body(const VS *x, VS *y, const GS *g, int64_t ncells, int kind, int64_t tile,
+                                             unsigned *status, StageBar *pb, unsigned st, const GS *gsm, int gcs,
+                                             unsigned char *smem_raw)
+{
+    metric_tile<N, CPB, Ar, VS, GS, STAGE, false, false, false, true, true>(
+        x, y, g, ncells, kind, batch_tab<N>(batch_tables<typename Ar::C>()), tile, CPB, smem_raw, nullptr, 0, nullptr,
+        nullptr, status, 0, pb, st, gsm, gcs);
+}
+
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
 __device__ __noinline__ void grouped_tile(const VS *x, VS *y, const GS *g, int64_t ncells, int kind, int64_t tile,
-                                          unsigned *status, const GS *gsm, int gcs, uint64_t *gbar, uint32_t gphase)
+                                          unsigned *status, StageBar *pb, unsigned st, const GS *gsm, int gcs)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    metric_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, batch_tab<N>(batch_tables<typename Ar::C>()), tile,
-                                           CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gcs, gbar, gphase);
+    grouped_body<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, pb, st, gsm, gcs, smem_raw);
 }
 
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
 __device__ __forceinline__ void grouped_one(const VS *x, VS *y, const GS *g, int64_t ncells, int kind, int64_t tile,
-                                            unsigned *status, const GS *gsm, int gcs, uint64_t *gbar, uint32_t gphase,
+                                            unsigned *status, StageBar *pb, unsigned st, const GS *gsm, int gcs,
                                             unsigned char *smem_raw)
 {
     if constexpr (std::is_same<Ar, ArDF>::value)
-        grouped_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, gsm, gcs, gbar, gphase);
+        grouped_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, pb, st, gsm, gcs);
     else
-        metric_tile<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, batch_tab<N>(batch_tables<typename Ar::C>()),
-                                               tile, CPB, smem_raw, nullptr, 0, nullptr, nullptr, status, 0, gsm, gcs,
-                                               gbar, gphase);
+        grouped_body<N, CPB, Ar, VS, GS, STAGE>(x, y, g, ncells, kind, tile, status, pb, st, gsm, gcs, smem_raw);
 }
 
 // ---- grouped mode: one persistent kernel per degree, shaped like the per-operator kernel
@@ -193,13 +201,16 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long s_next;
     __shared__ int s_prob;
-    // STAGE 1 layout: [line buffers][mbarrier, 16 B][metric tile]; STAGE 2: [line buffers][mbarrier]
+    // STAGE 1 layout: [line buffers][StageBar, 16 B][metric tile]; STAGE 2: [line buffers][StageBar]
     const size_t offb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), true>::RS * sizeof(T);  // a multiple of 16
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + offb);
-    GS *sG = reinterpret_cast<GS *>(smem_raw + offb + 16);
-    [[maybe_unused]] uint32_t phase = 0;  // of the barrier: flips with every staged tile
+    [[maybe_unused]] StageBar *sb = reinterpret_cast<StageBar *>(smem_raw + offb);
+    [[maybe_unused]] GS *sG = reinterpret_cast<GS *>(sb + 1);
+    [[maybe_unused]] unsigned phase = 0;  // kTilePhase of the next staged tile
     if (threadIdx.x == 0) {
-        if constexpr (STAGE != 0) mbar_init(bar, 1);  // once: it is live to the end of the CTA
+        if constexpr (STAGE != 0) {
+            mbar_init(&sb->bar, 1);  // once: it is live to the end of the CTA
+            sb->expired = 0;
+        }
         s_next = static_cast<long long>(atomicAdd(counter, 1ull));
     }
     for (;;) {
@@ -221,34 +232,42 @@ __global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb
         const int NC = metric_ncomp(P.kind);
         for (int64_t tile = t0; tile < t1; ++tile) {
             if (tile > t0) __syncthreads();  // the previous tile has finished with shared memory
-            bool staged = false;
+            bool staged = false;  // block-uniform
+            const unsigned stall = P.stall ? kTileStalled : 0u;
             if constexpr (STAGE == 1) {
                 const int64_t cell0 = tile * CPB;
                 const GS *gsrc = g + cell0 * NC * N3;
                 const uint32_t gb = CPB * NC * N3 * sizeof(GS);
-                staged = cell0 + CPB <= P.ncells && aligned16(gsrc) && gb % 16 == 0;  // block-uniform
+                staged = cell0 + CPB <= P.ncells && aligned16(gsrc) && gb % 16 == 0 && !sb->expired;
                 if (staged && threadIdx.x == 0) {  // waited for before the first right-hand side's physics
-                    mbar_expect_tx(bar, gb);
-                    metric_copy<CPB, PAD>(sG, gsrc, NC * N3, bar);
+                    mbar_expect_tx(&sb->bar, gb + (stall ? kStallBytes : 0u));
+                    metric_copy<CPB, PAD>(sG, gsrc, NC * N3, &sb->bar);
                 }
             }
+            bool again = false;
             for (int r = r0; r < r1; ++r) {
                 if (r > r0) __syncthreads();  // the previous right-hand side has finished with the line buffers
+                // the first right-hand side waits for the metric; if that wait ran out, the tile starts again
+                // without staging
+                again = STAGE == 1 && r == r0 + 1 && staged && sb->expired;
+                if (again) break;
                 const VS *x = static_cast<const VS *>(P.x) + r * P.stride;
                 VS *y = static_cast<VS *>(P.y) + r * P.stride;
                 if constexpr (STAGE == 1) {  // one code path: the metric from shared or from global memory
                     const GS *gm = staged ? sG : g + tile * CPB * NC * N3;
-                    grouped_one<N, CPB, Ar, VS, GS, 3>(x, y, g, P.ncells, P.kind, tile, P.status, gm,
-                                                       NC * N3 + (staged ? PAD : 0), staged && r == r0 ? bar : nullptr, phase, smem_raw);
+                    grouped_one<N, CPB, Ar, VS, GS, 3>(x, y, g, P.ncells, P.kind, tile, P.status,
+                                                       staged && r == r0 ? sb : nullptr, phase | stall, gm,
+                                                       NC * N3 + (staged ? PAD : 0), smem_raw);
                 } else {
-                    if constexpr (STAGE == 2) staged = x_tile_stageable<N, CPB>(x, tile * CPB, P.ncells);
-                    grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status, nullptr, 0,
-                                                           STAGE == 2 ? bar : nullptr, phase, smem_raw);
+                    if constexpr (STAGE == 2) staged = !sb->expired && x_tile_stageable<N, CPB>(x, tile * CPB, P.ncells);
+                    grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status,
+                                                           staged ? sb : nullptr, phase | stall, nullptr, 0, smem_raw);
                     // the next staged tile is copied over this one's line buffers, behind a barrier
                     if constexpr (STAGE == 2) fence_async_shared();
                 }
             }
-            if (staged) phase ^= 1u;
+            if (again) --tile;
+            else if (staged) phase ^= kTilePhase;
         }
     }
 }

@@ -74,7 +74,19 @@ __device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_c
 // short bound used when a test arms a barrier that cannot complete (see the fault-injection hook).
 constexpr uint32_t kWaitLimit = 1u << 22;
 constexpr uint32_t kWaitLimitInjected = 1u << 10;
+constexpr uint32_t kStallBytes = 16;  // what that hook arms beyond the copied bytes
 // bit set in an operator's device status word when a bounded wait expired
 constexpr unsigned kDevStatusTimeout = 1u;
+
+// The barrier of the tiles a persistent CTA stages one after another, in shared memory; initialised once. A
+// thread whose wait ran out sets `expired`: the CTA reads it behind the next barrier and stages nothing from
+// then on (the phase that did not complete leaves the barrier unusable, and its copy may still arrive).
+struct StageBar {
+    uint64_t bar;
+    uint32_t expired, unused;
+};
+// a staged tile's state, from the persistent loop to the tile's code
+constexpr unsigned kTilePhase = 1u;    // the phase it completes
+constexpr unsigned kTileStalled = 2u;  // the injected stall: short waits
 
 }  // namespace cw

@@ -61,3 +61,47 @@ def test_many_tiles_per_cta(cw, p, prec, kind):
                 assert ((y - ref).abs().max() <= 1e-6 * ref.abs().max()).item(), variant
     assert all(cw.cw_op_check(o.handle) == cw.CW_OK for o in ops)
     B.close()
+
+
+@pytest.mark.parametrize("prec", [0, 2], ids=["df64", "f32"])
+@pytest.mark.parametrize("p", [2, 3, 5])
+def test_expired_wait_ends_the_staging_of_its_cta(cw, p, prec):
+    """The batch's barriers armed with more bytes than the copies deliver: the waits run out. A metric tile is
+    read from global memory instead, for that and every later tile and right-hand side, so the results stay
+    right; an input tile gives zeros once per CTA, the later ones are read directly; both are reported, and a
+    batch without the injection on the same operators runs as always."""
+    import torch
+    ops, nrhs, xs, ys = big_batch(cw, prec, p, 1)
+    tol = 0.0 if prec == 0 else 1e-6  # as above
+    refs = [torch.cat([o.apply(x[r * o.L:(r + 1) * o.L].clone()) for r in range(n)])
+            for o, x, n in zip(ops, xs, nrhs)]
+    for variant in (2, 4):
+        for o in ops:
+            cw.cw_op_inject_stall(o.handle, True)
+        B = cw.Batch(ops, nrhs, xs, ys)
+        B.set_variant(p, variant)
+        for y in ys:
+            y.fill_(float("nan"))
+        B.launch()
+        assert cw.cw_op_check(ops[0].handle) == cw.CW_ERR_TIMEOUT
+        cw.cw_op_check(ops[1].handle)
+        y, ref = ys[0], refs[0]
+        assert torch.isfinite(y).all()
+        if variant == 2:
+            assert ((y - ref).abs().max() <= tol * ref.abs().max()).item()
+        else:  # at most one tile of zeros per resident CTA (16 a SM at the most)
+            cells = (y.view(nrhs[0], -1, (p + 1) ** 3) == 0).all(dim=2)
+            tile = B.variant(p)[1]
+            sms = torch.cuda.get_device_properties(0).multi_processor_count
+            assert 0 < int(cells.sum()) <= 16 * sms * tile
+            good = ~cells.unsqueeze(2).expand(-1, -1, (p + 1) ** 3).reshape(-1)
+            assert ((y - ref)[good].abs().max() <= tol * ref.abs().max()).item()
+        B.close()
+        for o in ops:
+            cw.cw_op_inject_stall(o.handle, False)
+        B = cw.Batch(ops, nrhs, xs, ys)
+        B.set_variant(p, variant)
+        B.launch()
+        assert cw.cw_op_check(ops[0].handle) == cw.CW_OK and cw.cw_op_check(ops[1].handle) == cw.CW_OK
+        assert ((ys[0] - refs[0]).abs().max() <= tol * refs[0].abs().max()).item()
+        B.close()
