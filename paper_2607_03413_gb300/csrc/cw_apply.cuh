@@ -537,6 +537,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
 {
     static_assert(!(RC && STAGE == 1), "recomputed geometry has no metric tile to stage");
     static_assert(PERSIST ? STAGE != 1 : STAGE != 3, "staging mode 3 is that of persistent callers");
+    static_assert(!(PERSIST && (SMOOTH || DOT)), "persistent callers apply the operator alone");
     // Double-float renormalisation of the intermediate values: kept where the operator serves the
     // solver (DOT), whose attainable accuracy depends on it (at 128^3 Q3 the double-float CG took
     // 1351 instead of 1026 iterations without it); skipped in the plain apply (5 % faster there,
@@ -572,6 +573,12 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
     // whole-line accesses of the input and output (LineVec) where they are wider than a value, but not at n = 6
     // in 8-byte vectors, where they cost the double-float kernel 6 % (Q5, 128e6 values: 33.3 -> 31.2 G values/s)
     constexpr bool WIDE = LineVec<N, VS>::WIDE && !(sizeof(VS) == 8 && N == 6);
+    // Lines are loaded (stored) whole before (after) their conversion, also where they are moved value by value.
+    // Not in the persistent tiles of n = 6 and 7, where the second copy of the line took the double-float function
+    // from 96 to 128 registers (n = 6; 16 right-hand sides on Q5 48^3 12.4 -> 11.2 ms together with the
+    // kernel's cap) and 178 to 128 (n = 7, 8 right-hand sides on Q6 24^3 1.58 -> 1.34 ms); at n = 5 it is faster with
+    // whole lines (Q4 40^3 1.73 against 1.75 ms), and so is the per-operator kernel (64^3 Q4 718 against 770 us).
+    constexpr bool LINES = WIDE || !PERSIST || N < 6;
     // load / store of a line of buffer R (0, 1, 2): x-line (own: the thread's own cell), y-line, z-pencil
     constexpr bool SW = tile_swizzled(N, sizeof(T), REMAP);
     using Z = TileSwz<N>;
@@ -702,22 +709,30 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         T v[N], w[N], u[N], acc[N], gx[N], gy[N], gz[N];
         // (1) x-line (j,k) = (ra, rb): N contiguous values of the cell, contracted with B along x
         {
-            VS xl[N];
-            bool have = act;
-            if (x_smem) {  // a thread whose wait expired reads nothing staged
-                have = x_ok;
-                if (x_ok) line_ld<N>(xs + N * r, xl, WIDE);
-            } else if (act) {
-                const VS *xg = x + cell * N3 + N * r;
-                if (WIDE && LineVec<N, VS>::aligned(x)) {
-                    LineVec<N, VS>::ld_nc(xg, xl);
-                } else {
+            const bool have = x_smem ? x_ok : act;  // a thread whose wait expired reads nothing staged
+            if constexpr (LINES) {
+                VS xl[N];
+                if (x_smem) {
+                    if (have) line_ld<N>(xs + N * r, xl, WIDE);
+                } else if (act) {
+                    const VS *xg = x + cell * N3 + N * r;
+                    if (WIDE && LineVec<N, VS>::aligned(x)) {
+                        LineVec<N, VS>::ld_nc(xg, xl);
+                    } else {
 #pragma unroll
-                    for (int m = 0; m < N; ++m) xl[m] = ldg_nc(xg + m);
+                        for (int m = 0; m < N; ++m) xl[m] = ldg_nc(xg + m);
+                    }
                 }
-            }
 #pragma unroll
-            for (int m = 0; m < N; ++m) v[m] = have ? Ar::from(xl[m]) : Ar::zero();
+                for (int m = 0; m < N; ++m) v[m] = have ? Ar::from(xl[m]) : Ar::zero();
+            } else if (x_smem) {
+#pragma unroll
+                for (int m = 0; m < N; ++m) v[m] = have ? Ar::from(xs[N * r + m]) : Ar::zero();
+            } else {
+                const VS *xg = x + (act ? cell : 0) * N3 + N * r;
+#pragma unroll
+                for (int m = 0; m < N; ++m) v[m] = have ? Ar::from(ldg_nc(xg + m)) : Ar::zero();
+            }
             sweep<N, Ar, 0, NRM>(tab, v, w);
             stx(0, true, w);
         }
@@ -936,38 +951,45 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
         {
             ldx(0, true, v);
             sweep<N, Ar, 1, NRM>(tab, v, w);
-            VS nv[N];  // the values to store
-            const bool yvec = WIDE && LineVec<N, VS>::aligned(y);
             const int64_t o = (act ? cell : 0) * N3 + N * r;
-#pragma unroll
-            for (int m = 0; m < N; ++m) Ar::to(nv[m], w[m]);
-            if constexpr (SMOOTH) {
-                VS yl[N], bl[N], dl[N];
-                line_ld<N>(y + o, yl, yvec);
-                line_ld<N>(sb + o, bl, LineVec<N, VS>::aligned(sb));
-                line_ld<N>(sd + o, dl, LineVec<N, VS>::aligned(sd));
-#pragma unroll
-                for (int m = 0; m < N; ++m) nv[m] = act ? yl[m] + dl[m] * (bl[m] - nv[m]) : VS(0);
-            }
-            if (SMOOTH || asm_nx > 0) {  // kernel-uniform: the x-interfaces inside the tile
-                // buffer 1 is free: its last reads precede the first barrier of step (5)
-                VS *exl = reinterpret_cast<VS *>(S0 + RS), *exr = exl + CPB * N2;
-                exl[c * N2 + r] = nv[0];
-                exr[c * N2 + r] = nv[N - 1];
-                __syncthreads();
+            if constexpr (!LINES) {  // (persistent callers neither assemble nor smooth)
                 if (act) {
-                    const int64_t ix = cell % asm_nx;
-                    if (c + 1 < cpt && cell + 1 < ncells && ix + 1 < asm_nx) {
-                        nv[N - 1] = AddOp<VS>::add(nv[N - 1], exl[(c + 1) * N2 + r]);
-                        if constexpr (SMOOTH) nv[N - 1] = nv[N - 1] * VS(0.5);
-                    }
-                    if (c > 0 && ix > 0) {
-                        nv[0] = AddOp<VS>::add(exr[(c - 1) * N2 + r], nv[0]);
-                        if constexpr (SMOOTH) nv[0] = nv[0] * VS(0.5);
+#pragma unroll
+                    for (int m = 0; m < N; ++m) Ar::to(y[o + m], w[m]);
+                }
+            } else {
+                VS nv[N];  // the values to store
+                const bool yvec = WIDE && LineVec<N, VS>::aligned(y);
+#pragma unroll
+                for (int m = 0; m < N; ++m) Ar::to(nv[m], w[m]);
+                if constexpr (SMOOTH) {
+                    VS yl[N], bl[N], dl[N];
+                    line_ld<N>(y + o, yl, yvec);
+                    line_ld<N>(sb + o, bl, LineVec<N, VS>::aligned(sb));
+                    line_ld<N>(sd + o, dl, LineVec<N, VS>::aligned(sd));
+#pragma unroll
+                    for (int m = 0; m < N; ++m) nv[m] = act ? yl[m] + dl[m] * (bl[m] - nv[m]) : VS(0);
+                }
+                if (SMOOTH || asm_nx > 0) {  // kernel-uniform: the x-interfaces inside the tile
+                    // buffer 1 is free: its last reads precede the first barrier of step (5)
+                    VS *exl = reinterpret_cast<VS *>(S0 + RS), *exr = exl + CPB * N2;
+                    exl[c * N2 + r] = nv[0];
+                    exr[c * N2 + r] = nv[N - 1];
+                    __syncthreads();
+                    if (act) {
+                        const int64_t ix = cell % asm_nx;
+                        if (c + 1 < cpt && cell + 1 < ncells && ix + 1 < asm_nx) {
+                            nv[N - 1] = AddOp<VS>::add(nv[N - 1], exl[(c + 1) * N2 + r]);
+                            if constexpr (SMOOTH) nv[N - 1] = nv[N - 1] * VS(0.5);
+                        }
+                        if (c > 0 && ix > 0) {
+                            nv[0] = AddOp<VS>::add(exr[(c - 1) * N2 + r], nv[0]);
+                            if constexpr (SMOOTH) nv[0] = nv[0] * VS(0.5);
+                        }
                     }
                 }
+                if (act) line_st<N>(y + o, nv, yvec);
             }
-            if (act) line_st<N>(y + o, nv, yvec);
         }
     }
 }

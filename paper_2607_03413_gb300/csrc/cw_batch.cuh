@@ -191,8 +191,15 @@ __device__ __forceinline__ void grouped_one(const VS *x, VS *y, const GS *g, int
 // R right-hand sides reads its metric from HBM once instead of R times; the right-hand sides' input is
 // read directly. STAGE 0 and 2: the per-operator kernel's modes, items (problem, chunk, right-hand
 // side) with the right-hand side fastest (the metric of a chunk read again from L2 for each).
+// Double-float at n = 6: capped to the 96 registers of the per-operator kernel (4 CTAs of 144 threads per SM, 3
+// with the 100 the loop and its tile take left alone: variant 0 of 16 right-hand sides on Q5 48^3 12.1 -> 11.1 ms).
+template <int N, int CPB, class Ar>
+constexpr int batch_min_blocks()
+{
+    return std::is_same<Ar, ArDF>::value && N == 6 ? 16 / CPB : 0;
+}
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
-__global__ void __launch_bounds__(N *N *CPB) batch_degree_kernel(const BatchProb *__restrict__ probs, int nprob,
+__global__ void __launch_bounds__(N *N *CPB, (batch_min_blocks<N, CPB, Ar>())) batch_degree_kernel(const BatchProb *__restrict__ probs, int nprob,
                                                                   int64_t nitems, unsigned long long *__restrict__ counter)
 {
     using T = typename Ar::T;
