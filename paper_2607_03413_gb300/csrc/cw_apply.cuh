@@ -963,12 +963,14 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
 #pragma unroll
                 for (int m = 0; m < N; ++m) Ar::to(nv[m], w[m]);
                 if constexpr (SMOOTH) {
-                    VS yl[N], bl[N], dl[N];
-                    line_ld<N>(y + o, yl, yvec);
-                    line_ld<N>(sb + o, bl, LineVec<N, VS>::aligned(sb));
-                    line_ld<N>(sd + o, dl, LineVec<N, VS>::aligned(sd));
+                    if (act) {  // (an idle slot must not read u of cell 0, which another CTA updates)
+                        VS yl[N], bl[N], dl[N];
+                        line_ld<N>(y + o, yl, yvec);
+                        line_ld<N>(sb + o, bl, LineVec<N, VS>::aligned(sb));
+                        line_ld<N>(sd + o, dl, LineVec<N, VS>::aligned(sd));
 #pragma unroll
-                    for (int m = 0; m < N; ++m) nv[m] = act ? yl[m] + dl[m] * (bl[m] - nv[m]) : VS(0);
+                        for (int m = 0; m < N; ++m) nv[m] = yl[m] + dl[m] * (bl[m] - nv[m]);
+                    }
                 }
                 if (SMOOTH || asm_nx > 0) {  // kernel-uniform: the x-interfaces inside the tile
                     // buffer 1 is free: its last reads precede the first barrier of step (5)
