@@ -504,9 +504,15 @@ static __device__ __noinline__ bool stage_wait_long_call(unsigned *status, Stage
 {
     return stage_wait_long(status, pb, st);
 }
-// Whether the copy behind a persistent CTA's barrier has arrived (bounded wait). INL: the double-float tile is a
-// function of its own, in the middle of which a call costs registers (n = 6: 128 instead of 103); in the FP32
-// body, inlined into the persistent loop, the code itself does (n = 8: 96 instead of 80).
+// Whether the long wait stands in the tile's code. The double-float tile is a function of its own, in the middle
+// of which a call costs registers (n = 6: 128 instead of 103). In FP32, 8 right-hand sides, inline / call: Q3 40^3 158 /
+// 153 us, Q1 64^3 132 / 124, but Q4 40^3 407 / 414 and, 16 of them, Q5 48^3 1932 / 1959.
+template <int N, class Ar>
+constexpr bool stage_wait_inline()
+{
+    return std::is_same<Ar, ArDF>::value || N == 5 || N == 6;
+}
+// Whether the copy behind a persistent CTA's barrier has arrived (bounded wait).
 template <bool INL>
 __device__ __forceinline__ bool stage_wait(unsigned *status, StageBar *pb, unsigned st)
 {
@@ -695,7 +701,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                 bulk_g2s(sX, xsrc, xb, bar);
             }
             if constexpr (PERSIST) {
-                x_ok = stage_wait<std::is_same<Ar, ArDF>::value>(status, pb, st);
+                x_ok = stage_wait<stage_wait_inline<N, Ar>()>(status, pb, st);
             } else {
                 x_ok = mbar_wait_bounded(bar, 0, lim);
                 if (!x_ok) wait_expired(status, bar, lim);
@@ -780,7 +786,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
             }
         } else if constexpr (STAGE == 3) {
             if (pb)  // block-uniform
-                g_ok = stage_wait<std::is_same<Ar, ArDF>::value>(status, pb, st);
+                g_ok = stage_wait<stage_wait_inline<N, Ar>()>(status, pb, st);
         }
         // (4) quadrature-point physics on the owned pencil, qp = (ra, rb, k)
         {
