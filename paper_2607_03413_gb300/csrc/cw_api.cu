@@ -879,7 +879,7 @@ cudaError_t apply_multi_launch(const Op *const *ops, const int64_t *off, int cou
     int64_t tiles = 0;
     for (int b = 0; b < count; ++b) {
         const Op &o = *ops[b];
-        one = one && o.geom == CW_GEOM_METRIC && o.stage == default_stage(o.n, f32) &&
+        one = one && o.geom == CW_GEOM_METRIC && o.stage == default_stage(o.n, f32, o.kind, o.E) &&
               o.cpb == (default_cells(o.n, f32, true) ? half : 0) &&
               o.E * (int64_t)(o.n * o.n) < ((int64_t)1 << 32);  // the fused x pass's interface numbers
         tiles += o.E;
@@ -1270,7 +1270,7 @@ cw_status cw_op_create(cw_mesh mh, int degree, int kind, int geom, int prec, int
     op->p = degree;
     op->n = degree + 1;
     if (geom == CW_GEOM_METRIC) {  // the variant to start with
-        if (prec == CW_PREC_F64) op->stage = default_stage(op->n, false);
+        if (prec == CW_PREC_F64) op->stage = default_stage(op->n, false, kind, m->ncells());
         if (default_cells(op->n, prec_f32_arith(prec), prec == CW_PREC_F32)) op->cpb = tile_cells(op->n, true) / 2;
     }
     op->kind = kind;

@@ -30,12 +30,24 @@ __host__ __device__ constexpr int tile_cells(int n, bool f32)
            : n == 6 ? (f32 ? 8 : 4) : n == 7 ? (f32 ? 8 : 4) : 2;
 }
 
-// Staging mode a stored-metric operator starts with (op.stage). FP32 arithmetic: 1 (input and metric
-// tiles by TMA). Double-float: 1, but 2 (metric prefetched into L2 and loaded in place) at n = 6 and 8, where
-// the staged metric's shared memory leaves 3 CTAs of 4 or 5 warps per SM. Laplace, mode 1 / 2 us: 51^3 Q5
-// 979 / 878, 35^3 Q7 699 / 684, but 99^3 Q2 471 / 502, 78^3 Q3 526 / 531, 64^3 Q4 K+M 790 / 798, 42^3 Q6
-// 785 / 838.
-__host__ __device__ constexpr int default_stage(int n, bool f32) { return !f32 && (n == 6 || n == 8) ? 2 : 1; }
+// Staging modes a stored-metric operator may start with: 1 (input and metric tiles by TMA), and in double-float at
+// n = 6 and 8 also 2 (metric prefetched into L2 and loaded in place), where the staged metric leaves 3 CTAs of 5 or 4
+// warps per SM and mode 2 runs 4 or 5.
+__host__ __device__ constexpr bool starts_in_two_stages(int n, bool f32) { return !f32 && (n == 6 || n == 8); }
+// The mode it starts with, by measurement (us, mode 1 / 2). The mass operator has one metric component and stays in
+// mode 1: Q5 103 / 107 at 8e6 entries, Q7 107 / 114. With the stiffness, mode 2 where mode 1 needs a second wave of
+// CTAs and its own slots do not (Q5 21.0 / 18.9, Q7 23.9 / 21.0 at 5e5 entries; but one wave 8.0 / 9.9 at 8e4) and, at
+// n = 6, from there on (Laplace 81 / 78 at 2e6, 280 / 254 at 8e6, 1115 / 985 at 3.3e7, with mass 82 / 80, 281 / 263, 1116 /
+// 1029). At n = 8 mode 1 stays ahead (Laplace 76 / 81 at 2e6, 140 / 144 at 4e6; with mass 268 / 277 at 8e6, 1076 / 1085
+// at 3.4e7) but for Laplace from 2^23 entries (265 / 263 at 8e6, 714 / 689 at 2.3e7, 1063 / 1024 at 3.4e7).
+inline int default_stage(int n, bool f32, int kind, int64_t cells)
+{
+    constexpr int64_t sms = 152;  // GB300
+    if (!starts_in_two_stages(n, f32) || kind == 2) return 1;
+    const int64_t tiles = (cells + tile_cells(n, f32) - 1) / tile_cells(n, f32);
+    if (n == 6) return tiles > 3 * sms ? 2 : 1;
+    return (tiles > 3 * sms && tiles <= 5 * sms) || (kind == 1 && cells >= 16384) ? 2 : 1;
+}
 // Whether a stored-metric operator starts with the alternative tile (half the default): FP32 vectors and
 // metric (g4) at n = 7, where 8 cells are 2 CTAs per SM (42^3 Q6 Laplace 175 us with 4 cells, 281 with 8; BF16
 // 182 with 8, 216 with 4). With a BF16 metric 4 cells would not do: their tile of 7 or 1 components is no

@@ -200,12 +200,12 @@ cudaError_t launch_metric(const Op &op, const void *x, void *y, cudaStream_t s, 
     return cudaGetLastError();
 }
 
-// several stored-metric operators in their default variant, at most kMultiOps per launch
-template <int N, class Ar, class VS, class GS>
-cudaError_t launch_multi(const Op *const *op, const int64_t *off, int count, const void *x, void *y, int *xtile,
+// several stored-metric operators in their default tile and staging mode ST, at most kMultiOps per launch
+template <int N, class Ar, class VS, class GS, int ST>
+cudaError_t launch_multi_st(const Op *const *op, const int64_t *off, int count, const void *x, void *y, int *xtile,
                          cudaStream_t s)
 {
-    constexpr int CPB = cpb_tuned<N, Ar, VS, GS, false>(), ST = default_stage(N, std::is_same<Ar, ArF32>::value);
+    constexpr int CPB = cpb_tuned<N, Ar, VS, GS, false>();
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op[0]->tab, [](double v) { return MakeC<Ar>::from(v); });
     const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op[0]->kind), ST);
@@ -228,6 +228,21 @@ cudaError_t launch_multi(const Op *const *op, const int64_t *off, int count, con
     return cudaSuccess;
 }
 
+// the staging mode the operators together start with
+template <int N, class Ar, class VS, class GS>
+cudaError_t launch_multi(const Op *const *op, const int64_t *off, int count, const void *x, void *y, int *xtile,
+                         cudaStream_t s)
+{
+    constexpr bool F32 = std::is_same<Ar, ArF32>::value;
+    if constexpr (starts_in_two_stages(N, F32)) {
+        int64_t cells = 0;
+        for (int b = 0; b < count; ++b) cells += op[b]->E;
+        if (default_stage(N, F32, op[0]->kind, cells) == 2)
+            return launch_multi_st<N, Ar, VS, GS, 2>(op, off, count, x, y, xtile, s);
+    }
+    return launch_multi_st<N, Ar, VS, GS, 1>(op, off, count, x, y, xtile, s);
+}
+
 template <class Ar, class VS, class GS>
 cudaError_t launch_multi_degree(const Op *const *op, const int64_t *off, int count, const void *x, void *y, int *xtile,
                                 cudaStream_t s)
@@ -244,13 +259,12 @@ cudaError_t launch_multi_degree(const Op *const *op, const int64_t *off, int cou
     return cudaErrorInvalidValue;
 }
 
-// One fused smoothing sweep (smooth_metric_kernel): default tile and staging; the x-interfaces inside tiles are averaged, *xfuse receives the
-// tile size for the x pass between tiles.
-template <int N, class Ar, class VS, class GS, bool RC>
-cudaError_t launch_smooth(const Op &op, void *u, const void *b, const void *dhat, cudaStream_t s, int *xfuse)
+// One fused smoothing sweep (smooth_metric_kernel): default tile, staging mode ST; the x-interfaces inside tiles are
+// averaged, *xfuse receives the tile size for the x pass between tiles.
+template <int N, class Ar, class VS, class GS, bool RC, int ST>
+cudaError_t launch_smooth_st(const Op &op, void *u, const void *b, const void *dhat, cudaStream_t s, int *xfuse)
 {
     constexpr int CPB = cpb_tuned<N, Ar, VS, GS, RC>();
-    constexpr int ST = RC ? 2 : default_stage(N, std::is_same<Ar, ArF32>::value);
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op.tab, [](double v) { return MakeC<Ar>::from(v); });
     const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op.kind), ST);
@@ -263,6 +277,15 @@ cudaError_t launch_smooth(const Op &op, void *u, const void *b, const void *dhat
                                          static_cast<const VS *>(dhat), static_cast<const GS *>(op.d_geo), op.E,
                                          op.kind, tab, op.mesh->nx, op.d_status, op.dbg_tma_extra);
     return cudaGetLastError();
+}
+
+// in the operator's staging mode where that is one of those it may start with, else the only such mode
+template <int N, class Ar, class VS, class GS, bool RC>
+cudaError_t launch_smooth(const Op &op, void *u, const void *b, const void *dhat, cudaStream_t s, int *xfuse)
+{
+    if constexpr (!RC && starts_in_two_stages(N, std::is_same<Ar, ArF32>::value))
+        if (op.stage == 2) return launch_smooth_st<N, Ar, VS, GS, RC, 2>(op, u, b, dhat, s, xfuse);
+    return launch_smooth_st<N, Ar, VS, GS, RC, RC ? 2 : 1>(op, u, b, dhat, s, xfuse);
 }
 
 template <class Ar, class VS, class GS>
@@ -286,12 +309,12 @@ cudaError_t launch_smooth_degree(const Op &op, void *u, const void *b, const voi
     return cudaErrorInvalidValue;
 }
 
-// y = A x with the CTA partials of <x, y> written to part (default tile size, TMA staging);
+// y = A x with the CTA partials of <x, y> written to part (default tile size, staging mode ST);
 // *nblocks receives the number of partials
-template <int N, class Ar, class VS, class GS, bool RC = false>
-cudaError_t launch_metric_dot(const Op &op, const void *x, void *y, double *part, int64_t *nblocks, cudaStream_t s)
+template <int N, class Ar, class VS, class GS, bool RC, int ST>
+cudaError_t launch_metric_dot_st(const Op &op, const void *x, void *y, double *part, int64_t *nblocks, cudaStream_t s)
 {
-    constexpr int CPB = cpb_tuned<N, Ar, VS, GS, RC>(), ST = RC ? 2 : default_stage(N, std::is_same<Ar, ArF32>::value);
+    constexpr int CPB = cpb_tuned<N, Ar, VS, GS, RC>();
     TabMetric<N, typename Ar::C> tab;
     fill_metric_tab<N>(tab, op.tab, [](double v) { return MakeC<Ar>::from(v); });
     const size_t smem = metric_smem_bytes<N, CPB, typename Ar::T, GS>(metric_ncomp(op.kind), ST);
@@ -304,6 +327,15 @@ cudaError_t launch_metric_dot(const Op &op, const void *x, void *y, double *part
                                          static_cast<const GS *>(op.d_geo), op.E, op.kind, tab, part, op.d_status,
                                          op.dbg_tma_extra);
     return cudaGetLastError();
+}
+
+// the staging mode as for the smoother
+template <int N, class Ar, class VS, class GS, bool RC>
+cudaError_t launch_metric_dot(const Op &op, const void *x, void *y, double *part, int64_t *nblocks, cudaStream_t s)
+{
+    if constexpr (!RC && starts_in_two_stages(N, std::is_same<Ar, ArF32>::value))
+        if (op.stage == 2) return launch_metric_dot_st<N, Ar, VS, GS, RC, 2>(op, x, y, part, nblocks, s);
+    return launch_metric_dot_st<N, Ar, VS, GS, RC, RC ? 2 : 1>(op, x, y, part, nblocks, s);
 }
 
 template <class Ar, class VS, class GS, bool RC>
