@@ -454,7 +454,7 @@ static cw_status coarse_setup(MgHier &h)
     CW_CUDA_TRY(cudaMemcpy(h.ainv, A.data(), A.size() * sizeof(double), cudaMemcpyHostToDevice));
     CW_CUDA_TRY(cudaMemcpy(h.rep, rep.data(), ni * sizeof(int), cudaMemcpyHostToDevice));
     CW_CUDA_TRY(cudaMemcpy(h.gi, gi.data(), op.L * sizeof(int), cudaMemcpyHostToDevice));
-    h.bytes += (int64_t)(A.size() + 2 * ni) * 8 + ni * 4 + op.L * 4 + op.L * (int64_t)h.es;
+    h.bytes += (int64_t)(A.size() + 2 * ni) * 8 + ni * 4 + op.L * 4;
     return CW_OK;
 }
 
