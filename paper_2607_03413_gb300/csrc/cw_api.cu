@@ -461,7 +461,7 @@ static bool dss_one_launch(const Op &op, int meshes)
     return op.p == 1 || op.L <= ((int64_t)1 << (meshes > 1 ? 21 : 19));
 }
 
-// one launch for `count` <= kDssMeshes meshes of one degree; xtile[b] as in dss_launch (0: none, -1: all)
+// one launch for `count` <= kDssMeshes meshes of one degree; xtile[b] as in dss_launch (0: none, -1: all; NULL: 0)
 template <class VS>
 static cudaError_t dss_node_typed(const Op *const *ops, const int64_t *off, const int *xtile, int count, VS *v,
                                   int flags, cudaStream_t s)
@@ -475,7 +475,8 @@ static cudaError_t dss_node_typed(const Op *const *ops, const int64_t *off, cons
         d.cta0 = cta;
         d.nodes = (uint32_t)(((int64_t)m.nx * ops[b]->p + 1) * ((int64_t)m.ny * ops[b]->p + 1) * ((int64_t)m.nz * ops[b]->p + 1));
         d.nx = m.nx, d.ny = m.ny, d.nz = m.nz;
-        d.xmask = xtile[b] < 0 ? -1 : xtile[b] > 1 ? xtile[b] - 1 : 0;  // tiles hold a power of two of cells
+        const int xt = xtile ? xtile[b] : 0;
+        d.xmask = xt < 0 ? -1 : xt > 1 ? xt - 1 : 0;  // tiles hold a power of two of cells
         d.fgx = FastDiv::make(m.nx * ops[b]->p + 1);
         d.fgy = FastDiv::make(m.ny * ops[b]->p + 1);
         cta += (d.nodes + 255) / 256;
@@ -835,13 +836,15 @@ cudaError_t dss_multi_launch(const Op *const *ops, const int64_t *off, const int
     const size_t es = vec_elem_size(ops[0]->prec);
     for (int b = 0; b < count;) {
         const int c = one ? std::min(count - b, kDssMeshes) : 1;
-        void *vb = static_cast<char *>(v) + off[b] * es;
+        const int *xt = xtile ? xtile + b : nullptr;
         cudaError_t e;
-        if (!one)
-            e = flags == CW_DSS_AVERAGE ? dss_average_launch(*ops[b], vb, s, xtile[b]) : dss_launch(*ops[b], vb, flags, s, xtile[b]);
-        else if (es == 8) e = dss_node_typed(ops + b, off + b, xtile + b, c, static_cast<double *>(v), flags, s);
-        else if (es == 4) e = dss_node_typed(ops + b, off + b, xtile + b, c, static_cast<float *>(v), flags, s);
-        else e = dss_node_typed(ops + b, off + b, xtile + b, c, static_cast<__nv_bfloat16 *>(v), flags, s);
+        if (!one) {
+            void *vb = static_cast<char *>(v) + off[b] * es;
+            e = flags == CW_DSS_AVERAGE ? dss_average_launch(*ops[b], vb, s, xt ? *xt : 0)
+                                        : dss_launch(*ops[b], vb, flags, s, xt ? *xt : 0);
+        } else if (es == 8) e = dss_node_typed(ops + b, off + b, xt, c, static_cast<double *>(v), flags, s);
+        else if (es == 4) e = dss_node_typed(ops + b, off + b, xt, c, static_cast<float *>(v), flags, s);
+        else e = dss_node_typed(ops + b, off + b, xt, c, static_cast<__nv_bfloat16 *>(v), flags, s);
         if (e != cudaSuccess) return e;
         b += c;
     }

@@ -143,7 +143,7 @@ cudaError_t apply_local(const Op &op, const void *x, void *y, cudaStream_t s, in
 // xtile > 0: the x pass skips the interfaces inside tiles of xtile consecutive cells (already summed)
 cudaError_t dss_launch(const Op &op, void *v, int flags, cudaStream_t s, int xtile = 0);
 // the same on `count` meshes of one degree and vector type whose vectors start at off[b] of v (one launch
-// for up to 16 small meshes)
+// for up to 16 small meshes); xtile may be NULL
 cudaError_t dss_multi_launch(const Op *const *ops, const int64_t *off, const int *xtile, int count, void *v, int flags,
                              cudaStream_t s);
 // y = A x on `count` operators of one degree, kind and precision whose vectors start at off[b] of x and y,

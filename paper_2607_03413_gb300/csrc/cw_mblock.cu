@@ -24,6 +24,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <new>
 #include <string>
 #include <unordered_map>
@@ -407,9 +408,8 @@ static cudaError_t mb_entities(const MBlock &mb, VS *v, cudaStream_t s)  // Algo
 template <class VS>
 static cudaError_t mb_dss_typed(const MBlock &mb, VS *v, int flags, const int *xtile, cudaStream_t s)
 {
-    const std::vector<int> none(mb.ops.size(), 0);
-    cudaError_t e = dss_multi_launch(mb.ops.data(), mb.off.data(), xtile ? xtile : none.data(), (int)mb.ops.size(), v,
-                                     CW_DSS_SUM, s);  // Algorithm struct_dss inside every block
+    cudaError_t e = dss_multi_launch(mb.ops.data(), mb.off.data(), xtile, (int)mb.ops.size(), v, CW_DSS_SUM,
+                                     s);  // Algorithm struct_dss inside every block
     if (e == cudaSuccess) e = mb_entities(mb, v, s);
     if (e != cudaSuccess) return e;
     if (flags == CW_DSS_AVERAGE)
@@ -634,9 +634,14 @@ cw_status cw_mblock_apply(cw_mblock h, const void *x, void *y, int flags, void *
     if (flags != CW_APPLY_LOCAL && flags != CW_APPLY_ASSEMBLE) return fail(CW_ERR_ARG, "cw_mblock_apply: bad flags");
     if (x == y) return fail(CW_ERR_ARG, "cw_mblock_apply: x and y must not alias");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    std::vector<int> xtile(mb->ops.size(), 0);
-    CW_CUDA_TRY(mb_apply_local(*mb, x, y, s, flags == CW_APPLY_ASSEMBLE ? xtile.data() : nullptr));
-    if (flags == CW_APPLY_ASSEMBLE) CW_CUDA_TRY(mb_dss(*mb, y, CW_DSS_SUM, s, xtile.data()));
+    if (flags == CW_APPLY_LOCAL) {
+        CW_CUDA_TRY(mb_apply_local(*mb, x, y, s));
+        return CW_OK;
+    }
+    const std::unique_ptr<int[]> xtile(new (std::nothrow) int[mb->ops.size()]());
+    if (!xtile) return fail(CW_ERR_OOM, "cw_mblock_apply: host allocation failed");
+    CW_CUDA_TRY(mb_apply_local(*mb, x, y, s, xtile.get()));
+    CW_CUDA_TRY(mb_dss(*mb, y, CW_DSS_SUM, s, xtile.get()));
     return CW_OK;
 }
 
