@@ -746,11 +746,28 @@ cudaError_t dss_from_f64(const Op &op, const double *src, double *dst, int flags
 // passes are bound by their FP64 additions and the one launch pays in large sums only: Q3 164/182, Q5
 // 147/162 at 32e6 entries, 43/42, 34/32 at 8e6, Q7 133/129; averages 239/184.
 template <class VS>
+constexpr bool dss_yz_built(int n, bool half)
+{
+    return sizeof(VS) < 8 ? n % 2 == 0 : !half && (n == 4 || n == 6);
+}
+template <class VS>
 static bool dss_yz_one_launch(const Op &op, int flags)
 {
-    if (op.n % 2 || (op.mesh->ny < 2 && op.mesh->nz < 2) || op.E * (2 * op.n - 1) >= ((int64_t)1 << 31)) return false;
-    if (sizeof(VS) < 8) return true;
-    return flags == CW_DSS_SUM && (op.n == 4 || op.n == 6) && op.L >= ((int64_t)1 << 24);
+    if (!dss_yz_built<VS>(op.n, flags == CW_DSS_AVERAGE) || (op.mesh->ny < 2 && op.mesh->nz < 2) ||
+        op.E * (2 * op.n - 1) >= ((int64_t)1 << 31))
+        return false;
+    return sizeof(VS) < 8 || op.L >= ((int64_t)1 << 24);
+}
+template <int N, bool HALF, class VS>
+static void dss_yz_launch(const Op &op, VS *v, cudaStream_t s)
+{
+    if constexpr (dss_yz_built<VS>(N, HALF)) {
+        const Mesh &m = *op.mesh;
+        const uint32_t nthr = (uint32_t)(op.E * (2 * N - 1));
+        dss_yz_kernel<N, VS, HALF><<<(nthr + 255) / 256, 256, 0, s>>>(
+            v, m.nx, m.ny, m.nz, nthr, FastDiv::make(2 * N - 1), FastDiv::make(m.nx), FastDiv::make(m.ny),
+            LineVec<N, VS>::aligned(v));
+    }
 }
 
 template <class VS>
@@ -769,14 +786,9 @@ static cudaError_t dss_typed(const Op &op, VS *v, int flags, cudaStream_t s, int
         const bool behind_x = first_axis == 0 && xtile == 0 && op.n == 4 && sizeof(VS) == 4 &&
                               op.L > ((int64_t)1 << 21) && op.L < ((int64_t)1 << 25);
         if (ax == 1 && end_axis == 3 && !behind_x && dss_yz_one_launch<VS>(op, flags)) {
-            const uint32_t nthr = (uint32_t)(op.E * (2 * op.n - 1));
             by_n(op.n, [&](auto N) {
-                const FastDiv fm = FastDiv::make(2 * N() - 1), fx = FastDiv::make(m.nx), fy = FastDiv::make(m.ny);
-                const bool vec = LineVec<N(), VS>::aligned(v);
-                if (flags == CW_DSS_AVERAGE)
-                    dss_yz_kernel<N(), VS, true><<<(nthr + 255) / 256, 256, 0, s>>>(v, m.nx, m.ny, m.nz, nthr, fm, fx, fy, vec);
-                else
-                    dss_yz_kernel<N(), VS, false><<<(nthr + 255) / 256, 256, 0, s>>>(v, m.nx, m.ny, m.nz, nthr, fm, fx, fy, vec);
+                if (flags == CW_DSS_AVERAGE) dss_yz_launch<N(), true>(op, v, s);
+                else dss_yz_launch<N(), false>(op, v, s);
             });
             break;
         }
