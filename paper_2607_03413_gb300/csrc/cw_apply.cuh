@@ -276,6 +276,35 @@ struct TileSwz {  // N = 4: a warp holds two cells (c odd and even); N = 8: half
     }
     static __host__ __device__ constexpr int D(int c) { return N == 4 ? 64 * c ^ ((c & 1) ? 24 : 0) : 512 * c; }
 };
+// The two claims above, for every warp of a tile: the words are a permutation of the buffer with each 16-byte
+// chunk of an x-line whole, and the accesses of 32 lanes (16-byte x accesses: of 8 lanes) cover every bank.
+template <int N, int CPB>
+constexpr bool tile_swz_ok()
+{
+    using Z = TileSwz<N>;
+    constexpr int N2 = N * N, SIZE = CPB * N2 * N;
+    bool seen[SIZE] = {};
+    for (int e = 0; e < SIZE; ++e) {
+        const int i = e % N, j = e / N % N, k = e / N2 % N, c = e / (N2 * N);
+        const int x = Z::D(c) ^ Z::B(j) ^ Z::C(k), w = x ^ Z::A(i);
+        if (w < 0 || w >= SIZE || seen[w] || w != (x ^ (i & ~3)) + (i & 3)) return false;
+        seen[w] = true;
+    }
+    for (int t0 = 0; t0 < CPB * N2; t0 += 32)
+        for (int m = 0; m < N; ++m) {
+            unsigned x[4] = {}, y = 0, z = 0;  // banks (of 8 lanes: 16-byte groups of banks) touched
+            for (int l = 0; l < 32; ++l) {
+                const int c = (t0 + l) / N2, ra = (t0 + l) % N, rb = (t0 + l) / N % N;
+                x[l / 8] |= 1u << ((Z::D(c) ^ Z::B(ra) ^ Z::C(rb) ^ (m & ~3)) / 4 % 8);
+                y |= 1u << ((Z::D(c) ^ Z::A(ra) ^ Z::C(rb) ^ Z::B(m)) % 32);
+                z |= 1u << ((Z::D(c) ^ Z::A(ra) ^ Z::B(rb) ^ Z::C(m)) % 32);
+            }
+            for (unsigned q : x)
+                if (q != 0xffu) return false;
+            if (y != 0xffffffffu || z != 0xffffffffu) return false;
+        }
+    return true;
+}
 struct TileGeom {
     int pi, pp, cs;  // row pitch, plane pitch, cell stride (elements)
     bool deal_x, deal_y;
@@ -587,6 +616,7 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
     constexpr bool LINES = WIDE || !PERSIST || N < 6;
     // load / store of a line of buffer R (0, 1, 2): x-line (own: the thread's own cell), y-line, z-pencil
     constexpr bool SW = tile_swizzled(N, sizeof(T), REMAP);
+    if constexpr (SW) static_assert(tile_swz_ok<N, CPB>(), "swizzled buffers: every word once, no bank conflict");
     using Z = TileSwz<N>;
     [[maybe_unused]] const int sx = Z::D(c) ^ Z::B(ra) ^ Z::C(rb), sy = Z::D(c) ^ Z::A(ra) ^ Z::C(rb);
     [[maybe_unused]] const int sz = Z::D(c) ^ Z::A(ra) ^ Z::B(rb);
