@@ -321,9 +321,9 @@ cw_status cw_cg_residual(cw_op op, const double *b, const double *u, int prec, d
  * problem with R right-hand sides reads its metric from HBM once, not R times); modes 0 and 2 are the
  * per-operator kernel's, per right-hand side. Mode
  * CW_BATCH_SINGLE: all degrees in ONE persistent kernel of 128-thread CTAs (variant = 0 full tile,
- * 1 half tile; items are (problem, chunk of tiles, right-hand side), right-hand side fastest); its 1D
- * tables live in the library's constant memory, uploaded at create, so only one single-mode batch per
- * precision may be launched at a time.
+ * 1 half tile; items are (problem, chunk of tiles, right-hand side), right-hand side fastest). The 1D
+ * tables of every degree live in the library's constant memory, uploaded at create with the same contents
+ * each time: batches of any degrees may exist and run together.
  */
 #define CW_BATCH_GROUPED 0
 #define CW_BATCH_SINGLE 1

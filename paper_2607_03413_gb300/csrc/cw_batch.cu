@@ -169,7 +169,6 @@ cw_status cw_batch_create(const cw_op *ops, const int *nrhs, const void *const *
     *out = nullptr;
     if (!ops || !nrhs || !x || !y || nprob < 1) return fail(CW_ERR_ARG, "cw_batch_create: NULL array or nprob < 1");
     Batch *b = new Batch;
-    const Tables1D *tabs[9] = {nullptr};
     std::vector<int> order(nprob);
     for (int i = 0; i < nprob; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
@@ -201,7 +200,6 @@ cw_status cw_batch_create(const cw_op *ops, const int *nrhs, const void *const *
         b->nrhs.push_back(nrhs[i]);
         b->x.push_back(x[i]);
         b->y.push_back(y[i]);
-        tabs[o->n] = &o->tab;
         b->tabs[o->n] = &o->tab;
     }
     // default variants: the per-operator kernel's default tile, the metric of a tile staged once for all right-hand
@@ -212,7 +210,7 @@ cw_status cw_batch_create(const cw_op *ops, const int *nrhs, const void *const *
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = b->fp64 ? batch_upload_tables_df(tabs) : batch_upload_tables_f32(tabs);
+    if (e == cudaSuccess) e = b->fp64 ? batch_upload_tables_df() : batch_upload_tables_f32();
     if (e == cudaSuccess) e = cudaMalloc(&b->d_probs, nprob * sizeof(BatchProb));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, 9 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);

@@ -308,8 +308,8 @@ inline size_t batch_smem_bytes(int n)
 }
 
 // per-unit entry points (cw_batch_df.cu: double-float on FP64 data; cw_batch_f32.cu: FP32)
-cudaError_t batch_upload_tables_df(const Tables1D *const tabs[9]);
-cudaError_t batch_upload_tables_f32(const Tables1D *const tabs[9]);
+cudaError_t batch_upload_tables_df();
+cudaError_t batch_upload_tables_f32();
 cudaError_t batch_launch_df(const BatchProb *d_probs, int nprob, int64_t nitems, unsigned long long *counter,
                             size_t smem, int grid, cudaStream_t s);
 cudaError_t batch_launch_f32(const BatchProb *d_probs, int nprob, int64_t nitems, unsigned long long *counter,

@@ -22,21 +22,28 @@ __global__ void __launch_bounds__(kBatchThreads, 4) batch_kernel_df(const BatchP
 static df64 mk(double v) { return df64{static_cast<float>(v), static_cast<float>(v - static_cast<double>(static_cast<float>(v)))}; }
 
 template <int N, class C>
-static void fill(TabMetric<N, C> &t, const Tables1D *tb)
+static void fill(TabMetric<N, C> &t)
 {
-    if (tb) fill_metric_tab<N>(t, *tb, mk);
+    Tables1D tb;
+    build_tables(N - 1, tb);
+    fill_metric_tab<N>(t, tb, mk);
 }
 
-cudaError_t batch_upload_tables_df(const Tables1D *const tabs[9])
+// The tables of every degree, whatever the batch's: they are the device's, for all batches together, so each
+// upload writes the same bytes (a batch that uploaded its own degrees' only would clear those of the others).
+cudaError_t batch_upload_tables_df()
 {
-    BatchTables<df64> h{};
-    fill<2>(h.t2, tabs[2]);
-    fill<3>(h.t3, tabs[3]);
-    fill<4>(h.t4, tabs[4]);
-    fill<5>(h.t5, tabs[5]);
-    fill<6>(h.t6, tabs[6]);
-    fill<7>(h.t7, tabs[7]);
-    fill<8>(h.t8, tabs[8]);
+    static const BatchTables<df64> h = [] {
+        BatchTables<df64> b{};
+        fill(b.t2);
+        fill(b.t3);
+        fill(b.t4);
+        fill(b.t5);
+        fill(b.t6);
+        fill(b.t7);
+        fill(b.t8);
+        return b;
+    }();
     return cudaMemcpyToSymbol(c_batch_tabs_df, &h, sizeof h);
 }
 
