@@ -67,9 +67,12 @@ def peaks():
 # dram__bytes_read.sum + dram__bytes_write.sum from one ncu capture per variant of a 40^3-cell case
 # (64,000 cells), to be scaled by the cell count of a launch. Variants not listed report null.
 DF64_KM_P4_TRAFFIC_PER_CELL = {
-    (8, 0): (512.066560e6 + 55.982592e6) / 64000,
-    (8, 2): (512.073984e6 + 55.491072e6) / 64000,
-    (4, 2): (512.065792e6 + 55.499776e6) / 64000,
+    (8, 0): (512.224512e6 + 55.667968e6) / 64000,
+    (8, 1): (512.056576e6 + 54.916352e6) / 64000,
+    (8, 2): (512.060672e6 + 55.767040e6) / 64000,
+    (4, 0): (512.129536e6 + 55.166976e6) / 64000,
+    (4, 1): (512.089088e6 + 54.504704e6) / 64000,
+    (4, 2): (512.060672e6 + 55.597312e6) / 64000,
 }
 
 # FP32 issue-rate roofline for double-float arithmetic: 152 SMs x 128 FP32 lanes x 2.07 GHz,

@@ -190,7 +190,8 @@ int64_t cw_op_device_bytes(cw_op op);
  * the two choices cw_op_get_variant reports -- and stage: 0 direct loads; 1 each CTA's input and
  * metric tiles moved into shared memory with bulk asynchronous copies (TMA) at kernel entry; 2 the
  * input tile by TMA and the metric tile prefetched into L2 by a bulk prefetch (less shared memory,
- * more CTAs per SM). An operator starts with the choice that measured fastest for its degree and precision. Results do not depend on the variant beyond rounding order. CW_PREC_F64_NATIVE has only
+ * more CTAs per SM). An operator starts with the choice that measured fastest for its degree, precision,
+ * kind and size. Results do not depend on the variant beyond rounding order. CW_PREC_F64_NATIVE has only
  * the default variant (CW_ERR_UNSUPPORTED otherwise). CW_GEOM_RECOMPUTE operators use the default
  * cells per CTA (another choice gives CW_ERR_UNSUPPORTED); stages 1 and 2 both stage the input
  * tile by TMA there (there is no metric tile).
@@ -315,7 +316,7 @@ cw_status cw_cg_residual(cw_op op, const double *b, const double *u, int prec, d
  * Work items are taken from a device counter by persistent CTAs (no waiting: an item number past the
  * end ends a CTA). Mode CW_BATCH_GROUPED (default): one persistent kernel per degree present, shaped
  * like the per-operator kernel (variant = cells-per-CTA choice + 2 * staging mode, 0..5; a batch starts with
- * the per-operator kernel's default); an item is a
+ * the per-operator kernel's default tile in mode 1, CW_PREC_F64 at degree 5 in mode 0); an item is a
  * (problem, chunk of tiles) pair and runs every right-hand side of the problem through each tile. With
  * staging mode 1 a tile's metric is moved into shared memory once and serves all right-hand sides (a
  * problem with R right-hand sides reads its metric from HBM once, not R times); modes 0 and 2 are the

@@ -450,7 +450,8 @@ __host__ __device__ constexpr int metric_ncomp(int kind) { return kind == 1 ? 6 
 // Line buffers of metric_tile: three for 4-byte elements; two for 8-byte ones (double-float and FP64
 // arithmetic), whose y-derivatives go back into buffer 0 after one more barrier: with the metric staged
 // a CTA then needs 72 instead of 80 bytes of shared memory per value (K+M), which is one more CTA per SM
-// at n = 5 and 8 (3 instead of 2).
+// at n = 5 and 8 (3 instead of 2). In modes 0 and 2, where shared memory is no limit, a third buffer in place of the
+// barrier changed nothing (Q5, 3e7 values: 1120 / 1118 us in mode 0, 924 / 922 in mode 2; batches within 1 %).
 template <class T>
 constexpr int line_buffers()
 {
@@ -1034,8 +1035,8 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
 
 // Register caps for the double-float kernels (as CTAs per SM for the launch bounds): stored metric
 // at n = 5 to 72 registers, which it fits without spilling, so that 4 CTAs of 200 threads fit per
-// SM (left alone the allocator takes 78 and loses one); recomputed geometry to 128 (2 CTAs at n = 5
-// instead of 1). Other n keep the plain kernel: larger n spill under a 72 cap, smaller n already fit
+// SM in staging modes 0 and 2 (left alone the allocator takes 78 and loses one; in mode 1, where it starts, shared
+// memory allows 3 either way); recomputed geometry to 128 (2 CTAs at n = 5 instead of 1). Other n keep the plain kernel: larger n spill under a 72 cap, smaller n already fit
 // and ran slower with the hint (a minimum-blocks hint is not neutral, even a hint of 1).
 template <class Ar, int N, bool RC>
 constexpr bool df_capped()

@@ -40,7 +40,7 @@ __host__ __device__ constexpr int batch_cpt(int N, int half)
 {
     return half ? (kBatchThreads / (N * N)) / 2 : kBatchThreads / (N * N);
 }
-// cell slots the 256 threads cover
+// cell slots the CTA's threads cover
 __host__ __device__ constexpr int batch_slots(int N) { return (kBatchThreads + N * N - 1) / (N * N); }
 
 struct BatchProb {
