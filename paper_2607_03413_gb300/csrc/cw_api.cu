@@ -473,7 +473,8 @@ static cudaError_t dss_node_typed(const Op *const *ops, const int64_t *off, cons
         DssMesh &d = tab.m[b];
         d.off = off ? off[b] : 0;
         d.cta0 = cta;
-        d.nodes = (uint32_t)(((int64_t)m.nx * ops[b]->p + 1) * ((int64_t)m.ny * ops[b]->p + 1) * ((int64_t)m.nz * ops[b]->p + 1));
+        const int64_t p = ops[b]->p;
+        d.nodes = (uint32_t)((m.nx * p + 1) * (m.ny * p + 1) * (m.nz * p + 1));
         d.nx = m.nx, d.ny = m.ny, d.nz = m.nz;
         const int xt = xtile ? xtile[b] : 0;
         d.xmask = xt < 0 ? -1 : xt > 1 ? xt - 1 : 0;  // tiles hold a power of two of cells

@@ -482,7 +482,8 @@ template <int N, int CPB, class T, class GS, bool REMAP = true>
 __host__ __device__ constexpr size_t metric_smem_bytes(int nc, int stage)
 {
     constexpr size_t lb = line_buffers<T>() * TileLines<N, CPB, sizeof(T), REMAP>::RS * sizeof(T);  // a multiple of 16
-    return stage == 1 ? lb + (CPB * (nc * N * N * N + metric_pad<N, T, GS>()) * sizeof(GS) + 15) / 16 * 16 + 16 : stage == 2 ? lb + 16 : lb;
+    const size_t metric = (CPB * (nc * N * N * N + metric_pad<N, T, GS>()) * sizeof(GS) + 15) / 16 * 16;
+    return stage == 1 ? lb + metric + 16 : stage == 2 ? lb + 16 : lb;
 }
 
 // whether a whole tile of CPB cells can be moved by one bulk copy from vector x (16-byte alignment and size)
@@ -504,8 +505,8 @@ __device__ __forceinline__ bool x_tile_stageable(const VS *x, int64_t cell0, int
 // are left to the DSS.
 // RC: geo holds the trilinear coefficients (kTriCoef per cell) and the metric of every quadrature
 // point is recomputed from them (Sec. 6: J, det J, J^-1 at the point), G = (w / det J) [c_a . c_b], applied
-// without forming it: G g = (w / det J) c_a . (sum_b c_b g_b), with c_0 = J_eta x J_zeta, c_1 = J_zeta x J_xi, c_2 = J_xi x J_eta (the rows of det J J^-1), and
-// the mass coefficient w det J.
+// without forming it: G g = (w / det J) c_a . (sum_b c_b g_b), with c_0 = J_eta x J_zeta, c_1 = J_zeta x J_xi,
+// c_2 = J_xi x J_eta (the rows of det J J^-1), and the mass coefficient w det J.
 // SMOOTH (Algorithm smoother_fused in one pass over the operator's output): y aliases x (= u, updated
 // in place), and the stored value is u + D_hat (b - A u) (sb = b, sd = D_hat, cell-wise in the vector
 // type), with the x-interfaces inside the tile averaged (the x pass of the averaging DSS:
@@ -535,8 +536,8 @@ static __device__ __noinline__ bool stage_wait_long_call(unsigned *status, Stage
     return stage_wait_long(status, pb, st);
 }
 // Whether the long wait stands in the tile's code. The double-float tile is a function of its own, in the middle
-// of which a call costs registers (n = 6: 128 instead of 103). In FP32, 8 right-hand sides, inline / call: Q3 40^3 158 /
-// 153 us, Q1 64^3 132 / 124, but Q4 40^3 407 / 414 and, 16 of them, Q5 48^3 1932 / 1959.
+// of which a call costs registers (n = 6: 128 instead of 103). In FP32, 8 right-hand sides, inline / call: Q3 40^3
+// 158 / 153 us, Q1 64^3 132 / 124, but Q4 40^3 407 / 414 and, 16 of them, Q5 48^3 1932 / 1959.
 template <int N, class Ar>
 constexpr bool stage_wait_inline()
 {
@@ -898,7 +899,8 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
                     cmr = Ar::norm(Ar::mul(w, det));
                     if (HAS_K) {
                         // h_a = (w / det J) c_a . v with v = sum_b c_b g_b: 18 multiply-adds and 3 scalings
-                        // where forming G first takes 27 and 6 (41x40x39 Q4 K+M 449 -> 419 us, error 2.8e-14 -> 1.8e-14)
+                        // where forming G first takes 27 and 6 (41x40x39 Q4 K+M 449 -> 419 us, error 2.8e-14 ->
+                        // 1.8e-14)
                         const T sc = Ar::div(w, det);
                         T vv[3];
 #pragma unroll
@@ -1036,8 +1038,9 @@ __device__ __forceinline__ void metric_tile(const VS *x, VS *y, const GS *__rest
 // Register caps for the double-float kernels (as CTAs per SM for the launch bounds): stored metric
 // at n = 5 to 72 registers, which it fits without spilling, so that 4 CTAs of 200 threads fit per
 // SM in staging modes 0 and 2 (left alone the allocator takes 78 and loses one; in mode 1, where it starts, shared
-// memory allows 3 either way); recomputed geometry to 128 (2 CTAs at n = 5 instead of 1). Other n keep the plain kernel: larger n spill under a 72 cap, smaller n already fit
-// and ran slower with the hint (a minimum-blocks hint is not neutral, even a hint of 1).
+// memory allows 3 either way); recomputed geometry to 128 (2 CTAs at n = 5 instead of 1). Other n keep the plain
+// kernel: larger n spill under a 72 cap, smaller n already fit and ran slower with the hint (a minimum-blocks hint
+// is not neutral, even a hint of 1).
 template <class Ar, int N, bool RC>
 constexpr bool df_capped()
 {

@@ -203,8 +203,9 @@ cw_status cw_batch_create(const cw_op *ops, const int *nrhs, const void *const *
         b->tabs[o->n] = &o->tab;
     }
     // default variants: the per-operator kernel's default tile, the metric of a tile staged once for all right-hand
-    // sides; but in double-float at n = 6 direct loads, which leave 4 CTAs per SM instead of 3 (us, mode 0 / 1 / 2: 16
-    // right-hand sides on Q5 48^3 11100 / 12200 / 11230, one on 24^3 107 / 116 / 110; n = 8, 2 on Q7 24^3 555 / 485 / 509)
+    // sides; but in double-float at n = 6 direct loads, which leave 4 CTAs per SM instead of 3 (us, mode 0 / 1 / 2:
+    // 16 right-hand sides on Q5 48^3 11100 / 12200 / 11230, one on 24^3 107 / 116 / 110; n = 8, 2 on Q7 24^3 555 / 485 /
+    // 509)
     for (int n = 2; n <= 8; ++n)
         b->variant[n] = (b->fp64 && n == 6 ? 0 : 2) + (default_cells(n, !b->fp64, true) ? 1 : 0);
     int dev = 0;

@@ -199,8 +199,9 @@ constexpr int batch_min_blocks()
     return std::is_same<Ar, ArDF>::value && N == 6 ? 16 / CPB : 0;
 }
 template <int N, int CPB, class Ar, class VS, class GS, int STAGE>
-__global__ void __launch_bounds__(N *N *CPB, (batch_min_blocks<N, CPB, Ar>())) batch_degree_kernel(const BatchProb *__restrict__ probs, int nprob,
-                                                                  int64_t nitems, unsigned long long *__restrict__ counter)
+__global__ void __launch_bounds__(N *N *CPB, (batch_min_blocks<N, CPB, Ar>()))
+    batch_degree_kernel(const BatchProb *__restrict__ probs, int nprob, int64_t nitems,
+                        unsigned long long *__restrict__ counter)
 {
     using T = typename Ar::T;
     constexpr int N3 = N * N * N;
@@ -266,7 +267,8 @@ __global__ void __launch_bounds__(N *N *CPB, (batch_min_blocks<N, CPB, Ar>())) b
                                                        staged && r == r0 ? sb : nullptr, phase | stall, gm,
                                                        NC * N3 + (staged ? PAD : 0), smem_raw);
                 } else {
-                    if constexpr (STAGE == 2) staged = !sb->expired && x_tile_stageable<N, CPB>(x, tile * CPB, P.ncells);
+                    if constexpr (STAGE == 2)
+                        staged = !sb->expired && x_tile_stageable<N, CPB>(x, tile * CPB, P.ncells);
                     grouped_one<N, CPB, Ar, VS, GS, STAGE>(x, y, g, P.ncells, P.kind, tile, P.status,
                                                            staged ? sb : nullptr, phase | stall, nullptr, 0, smem_raw);
                     // the next staged tile is copied over this one's line buffers, behind a barrier

@@ -604,7 +604,8 @@ static bool apply_dot_ok(const Op &op, int ak)
     if (op.geom == CW_GEOM_METRIC ? op.stage != 1 && !(op.stage == 2 && starts_in_two_stages(op.n, f32))
                                   : op.geom != CW_GEOM_RECOMPUTE)
         return false;
-    if (op.cpb != 0 && !(op.geom == CW_GEOM_METRIC && default_cells(op.n, f32, op.prec == CW_PREC_F32))) return false;  // not the default tile
+    if (op.cpb != 0 && !(op.geom == CW_GEOM_METRIC && default_cells(op.n, f32, op.prec == CW_PREC_F32)))
+        return false;  // not the default tile
     return op.prec == CW_PREC_F64 || op.prec == CW_PREC_F32 || op.prec == CW_PREC_F32_BF16G;
 }
 

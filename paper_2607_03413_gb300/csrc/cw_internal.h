@@ -36,10 +36,10 @@ __host__ __device__ constexpr int tile_cells(int n, bool f32)
 __host__ __device__ constexpr bool starts_in_two_stages(int n, bool f32) { return !f32 && (n == 6 || n == 8); }
 // The mode it starts with, by measurement (us, mode 1 / 2). The mass operator has one metric component and stays in
 // mode 1: Q5 103 / 107 at 8e6 entries, Q7 107 / 114. With the stiffness, mode 2 where mode 1 needs a second wave of
-// CTAs and its own slots do not (Q5 21.0 / 18.9, Q7 23.9 / 21.0 at 5e5 entries; but one wave 8.0 / 9.9 at 8e4) and, at
-// n = 6, from there on (Laplace 81 / 78 at 2e6, 280 / 254 at 8e6, 1115 / 985 at 3.3e7, with mass 82 / 80, 281 / 263, 1116 /
-// 1029). At n = 8 mode 1 stays ahead (Laplace 76 / 81 at 2e6, 140 / 144 at 4e6; with mass 268 / 277 at 8e6, 1076 / 1085
-// at 3.4e7) but for Laplace from 2^23 entries (265 / 263 at 8e6, 714 / 689 at 2.3e7, 1063 / 1024 at 3.4e7).
+// CTAs and its own slots do not (Q5 21.0 / 18.9, Q7 23.9 / 21.0 at 5e5 entries; but one wave 8.0 / 9.9 at 8e4) and,
+// at n = 6, from there on (Laplace 81 / 78 at 2e6, 280 / 254 at 8e6, 1115 / 985 at 3.3e7, with mass 82 / 80, 281 / 263,
+// 1116 / 1029). At n = 8 mode 1 stays ahead (Laplace 76 / 81 at 2e6, 140 / 144 at 4e6; with mass 268 / 277 at 8e6,
+// 1076 / 1085 at 3.4e7) but for Laplace from 2^23 entries (265 / 263 at 8e6, 714 / 689 at 2.3e7, 1063 / 1024 at 3.4e7).
 inline int default_stage(int n, bool f32, int kind, int64_t cells)
 {
     constexpr int64_t sms = 152;  // GB300

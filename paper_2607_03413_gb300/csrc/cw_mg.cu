@@ -203,8 +203,8 @@ static bool fused_sweep(const MgHier &h, const Op &op)
 }
 
 // `sweeps` sweeps of Algorithm smoother_fused: u <- S_bar (u + D_hat (b - A u)). The first sweep from
-// u = 0 (zero) is u = S_bar D_hat b, the product formed in the first averaging pass. A fused sweep is one operator launch whose epilogue applies the
-// update and the x averages inside its tiles, then the x pass between tiles and the y and z passes of
+// u = 0 (zero) is u = S_bar D_hat b, the product formed in the first averaging pass. A fused sweep is one
+// operator launch whose epilogue applies the update and the x averages inside its tiles, then the x pass between tiles and the y and z passes of
 // the averaging DSS; otherwise operator, update kernel and the three averaging passes.
 template <class VS>
 static cudaError_t smooth_t(const MgHier &h, int l, const VS *b, VS *u, int sweeps, bool zero, cudaStream_t s)
